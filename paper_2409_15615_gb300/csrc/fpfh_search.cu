@@ -15,9 +15,9 @@
 //                          tau_num and tau_lin (step 1)
 //   valid_walk             |I_valid(q)| over the neighbours with B; J (step 2)
 //   spfh_walk, fpfh_walk   over B neighbours, for B points / for J
-// The normals take one thread per query on a large cloud and one warp per
-// query on a small one, by the same rule as kmx_normals (kThreadQueryMin);
-// the other stages take one warp per query.  Queries run in the grid's cell
+// The normals take one lane per query on a large cloud and one warp per query
+// on a small one, by the same rule and with the same code as kmx_normals
+// (kThreadQueryMin); the other stages take one warp per query.  Queries run in the grid's cell
 // order so that neighbouring threads and warps walk the same cells.  The neighbours a stage visits come
 // in the same order as in the stored lists of kmx_normals, so every sum is
 // formed in the same order and the list-free Faster-PFH reproduces the
@@ -58,42 +58,58 @@ ClassicScratch carve(void* base, int64_t n, bool need_spfh, size_t* total)
 // Faster-PFH (step 1): also |I(q)| over r_FPFH; PCA when |I| >= tau_num and
 // |P_normal| >= tau_num; bit0 = B (normal and p_lin < tau_lin).  bit2 = PCA.
 template <bool kClassic>
+__device__ __forceinline__ void store_normal(float4 q, int nf, int nn, const float* mom, const float* vp, int tau_num,
+                                             float tau_lin, float4* __restrict__ normal4, uint8_t* __restrict__ flags,
+                                             int32_t* __restrict__ jflag)
+{
+    const int qi = __float_as_int(q.w);
+    uint8_t flag = 0;
+    float4 nout = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (kClassic ? nn >= kMinNormal : (nf >= tau_num && nn >= tau_num)) {
+        double plin;
+        flag |= 4;
+        const bool has = normal_from_moments(mom, nn, q.x, q.y, q.z, vp, &nout, &plin);
+        if (kClassic && has) flag |= 3;
+        if (!kClassic && has && plin < (double)tau_lin) flag |= 1;
+    }
+    normal4[qi] = nout;
+    flags[qi] = flag;
+    if (kClassic) jflag[qi] = flag & 1;
+}
+
+// Large clouds: 32 queries per warp, one per lane (the sums of kmx_normals, so
+// the same bits).
+template <bool kClassic>
+__global__ void __launch_bounds__(32 * kLaneWarps, 6)
+    lane_normals(GridView g, Radii R, float vp0, float vp1, float vp2, int tau_num, float tau_lin,
+                 float4* __restrict__ normal4, uint8_t* __restrict__ flags, int32_t* __restrict__ jflag)
+{
+    __shared__ LaneQueries sm[kLaneWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t n_sorted = *g.n_sorted;
+    const float vp[3] = {vp0, vp1, vp2};
+    if (n_sorted < kThreadQueryMin) return;
+    for_each_batch(g, (int64_t)blockIdx.x * kLaneWarps + warp, (int64_t)gridDim.x * kLaneWarps, lane,
+                   [&](float4 q, int nq, int start, int excl, int total) {
+                       int nf, nn;
+                       float mom[9];
+                       lane_moments(g, R, start, excl, total, nq, lane, sm[warp], q, &nf, &nn, mom);
+                       if (lane < nq) store_normal<kClassic>(q, nf, nn, mom, vp, tau_num, tau_lin, normal4, flags, jflag);
+                   });
+}
+
+template <bool kClassic>
 __global__ void __launch_bounds__(kThreads) walk_normals(GridView g, Radii R, float vp0, float vp1, float vp2,
                                                          int tau_num, float tau_lin, float4* __restrict__ normal4,
                                                          uint8_t* __restrict__ flags, int32_t* __restrict__ jflag)
 {
     __shared__ float sm_mom[9][kQPerBlock];
     __shared__ float sm_q[3][kQPerBlock];
-    __shared__ int sm_qi[kQPerBlock], sm_nN[kQPerBlock];
+    __shared__ int sm_qi[kQPerBlock], sm_nF[kQPerBlock], sm_nN[kQPerBlock];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t n_sorted = *g.n_sorted;
     const float vp[3] = {vp0, vp1, vp2};
-    if (n_sorted >= kThreadQueryMin) {
-        // one thread per query: the two sweeps of kmx_normals (the same
-        // order, so the same bits), then the FP64 solve of its moments
-        for (int64_t p = (int64_t)blockIdx.x * kThreads + threadIdx.x; p < n_sorted; p += (int64_t)gridDim.x * kThreads) {
-            const float4 q = g.sorted[p];
-            const int qi = __float_as_int(q.w);
-            const Sweep1 r = sweep1(g, R, p, q);
-            const bool pca = kClassic ? r.nn >= kMinNormal : (r.nf >= tau_num && r.nn >= tau_num);
-            uint8_t flag = 0;
-            float4 nout = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (pca) {
-                const float inv = r.nn > 0 ? 1.0f / (float)r.nn : 0.0f;
-                float mom[9];
-                sweep2(g, R, p, q, r.sx * inv, r.sy * inv, r.sz * inv, mom, nullptr);
-                double plin;
-                flag |= 4;
-                const bool has = normal_from_moments(mom, r.nn, q.x, q.y, q.z, vp, &nout, &plin);
-                if (kClassic && has) flag |= 3;
-                if (!kClassic && has && plin < (double)tau_lin) flag |= 1;
-            }
-            normal4[qi] = nout;
-            flags[qi] = flag;
-            if (kClassic) jflag[qi] = flag & 1;
-        }
-        return;
-    }
+    if (n_sorted >= kThreadQueryMin) return;  // lane_normals
     // one warp per query (the same layout as kmx_normals on a small cloud);
     // the block's 32 queries are solved by warp 0, one per lane
     // uniform over the block: every thread reaches the barriers
@@ -188,29 +204,17 @@ __global__ void __launch_bounds__(kThreads) walk_normals(GridView g, Radii R, fl
                 sm_q[1][slot] = q.y;
                 sm_q[2][slot] = q.z;
                 sm_qi[slot] = __float_as_int(q.w);
-                sm_nN[slot] = pca ? nn : -1;
+                sm_nF[slot] = nf;
+                sm_nN[slot] = nn;
             }
         }
         __syncthreads();
         if (warp == 0 && sm_qi[lane] >= 0) {
-            const int qi = sm_qi[lane];
-            const int nN = sm_nN[lane];
-            uint8_t flag = 0;
-            float4 nout = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (nN >= 0) {
-                float mom[9];
+            float mom[9];
 #pragma unroll
-                for (int i = 0; i < 9; ++i) mom[i] = sm_mom[i][lane];
-                double plin;
-                flag |= 4;
-                const bool has = normal_from_moments(mom, nN, sm_q[0][lane], sm_q[1][lane], sm_q[2][lane], vp, &nout,
-                                                     &plin);
-                if (kClassic && has) flag |= 3;
-                if (!kClassic && has && plin < (double)tau_lin) flag |= 1;
-            }
-            normal4[qi] = nout;
-            flags[qi] = flag;
-            if (kClassic) jflag[qi] = flag & 1;
+            for (int i = 0; i < 9; ++i) mom[i] = sm_mom[i][lane];
+            store_normal<kClassic>(make_float4(sm_q[0][lane], sm_q[1][lane], sm_q[2][lane], __int_as_float(sm_qi[lane])),
+                                   sm_nF[lane], sm_nN[lane], mom, vp, tau_num, tau_lin, normal4, flags, jflag);
         }
         __syncthreads();  // the shared moments are rewritten by the next chunk
     }
@@ -395,11 +399,7 @@ cudaError_t kmx_fpfh_search_launch(kmx_ctx* ctx, const kmx_grid* g, const kmx_pa
     ClassicScratch s = carve(scratch, g->n_cap, spfh == nullptr, &total);
     float* sp = spfh ? spfh : s.spfh;
     GridView gv{g->sorted, g->cells, g->keys, g->table_size, g->inv_cell, g->d_n_sorted, g->sslot};
-    Radii R;
-    R.rf2 = prm->r_fpfh * prm->r_fpfh;
-    R.rn2 = prm->r_normal * prm->r_normal;
-    R.rf2d = (double)prm->r_fpfh * (double)prm->r_fpfh;
-    R.rn2d = (double)prm->r_normal * (double)prm->r_normal;
+    const Radii R = make_radii(prm);
     const int64_t n = g->n_cap;
     cudaError_t e;
     // points outside the bucketed set (only after a range error) keep zeros
@@ -410,6 +410,14 @@ cudaError_t kmx_fpfh_search_launch(kmx_ctx* ctx, const kmx_grid* g, const kmx_pa
     const unsigned nbn = kmx_stride_blocks(n, kQPerBlock, ctx->sm_count);
     const unsigned nbw = kmx_stride_blocks(n, kWarps, ctx->sm_count);
     const float4* n4 = reinterpret_cast<const float4*>(normal4);
+    const unsigned nbl = kmx_stride_blocks(n, 32 * kLaneWarps, ctx->sm_count, 32);
+    const bool large = n >= kThreadQueryMin;  // the device count may be
+    if (large) {
+        KMX_COUNT_LAUNCH();
+        (classic ? lane_normals<true> : lane_normals<false>)<<<nbl, 32 * kLaneWarps, 0, st>>>(
+            gv, R, prm->viewpoint[0], prm->viewpoint[1], prm->viewpoint[2], prm->tau_num, prm->tau_lin,
+            reinterpret_cast<float4*>(normal4), flags, s.jflag);
+    }
     KMX_COUNT_LAUNCH();
     if (classic) {
         walk_normals<true><<<nbn, kThreads, 0, st>>>(gv, R, prm->viewpoint[0], prm->viewpoint[1], prm->viewpoint[2],

@@ -27,7 +27,20 @@ struct GridView {
 struct Radii {
     float rf2, rn2;     // FP32 squared radii
     double rf2d, rn2d;  // FP64 squared radii, (double)r * (double)r
+    float ef, en;       // half-widths of the bands around them in which FP64 decides (within)
 };
+
+inline Radii make_radii(const kmx_params* prm)
+{
+    Radii R;
+    R.rf2 = prm->r_fpfh * prm->r_fpfh;
+    R.rn2 = prm->r_normal * prm->r_normal;
+    R.rf2d = (double)prm->r_fpfh * (double)prm->r_fpfh;
+    R.rn2d = (double)prm->r_normal * (double)prm->r_normal;
+    R.ef = 1e-5f * R.rf2;
+    R.en = 1e-5f * R.rn2;
+    return R;
+}
 
 // Is a within radius of q?  FP32 unless the FP32 distance lies within 1e-5
 // (relative) of r^2, where the FP64 expression ((dx*dx + dy*dy) + dz*dz) <
@@ -90,104 +103,6 @@ __device__ __forceinline__ int stencil(const GridView& g, int64_t p, int lane, i
     return stencil_at(g, cx, cy, cz, lane, start, excl);
 }
 
-// The stencil of the last query a warp searched, reused while the next
-// queries (consecutive in cell order) sit in the same cell.
-struct StencilCache {
-    unsigned long long key = KMX_EMPTY_KEY;
-    int start = 0, excl = 0, total = 0;
-
-    __device__ __forceinline__ int get(const GridView& g, int64_t p, int lane)
-    {
-        const unsigned long long k = cell_key_at(g, p);
-        if (k != key) {
-            int x, y, z;
-            unpack_cell(k, &x, &y, &z);
-            total = stencil_at(g, x, y, z, lane, &start, &excl);
-            key = k;
-        }
-        return total;
-    }
-};
-
-// Device point count from which the radius searches (normals, the list-free
-// FPFH path) give each query one thread; below it one warp takes a query, so
-// that a small cloud still fills the GPU.  Every search kernel applies the
-// same rule, which keeps the list and list-free paths bit-identical.
-constexpr int64_t kThreadQueryMin = 65536;
-
-// One thread per query: calls f(a) for every bucketed point a of the 27-cell
-// stencil around sorted position p, in the order of the stored neighbour
-// lists (cells dx fastest, then dy, then dz; points of a cell in sorted
-// order).
-template <typename F>
-__device__ __forceinline__ void for_each_candidate(const GridView& g, int64_t p, F&& f)
-{
-    int cx, cy, cz;
-    unpack_cell(cell_key_at(g, p), &cx, &cy, &cz);
-    for (int c = 0; c < 27; ++c) {
-        const int dx = c % 3 - 1, dy = (c / 3) % 3 - 1, dz = c / 9 - 1;
-        const int slot = kmx_hash_find(g.keys, g.T, kmx_pack_key(cx + dx, cy + dy, cz + dz));
-        if (slot < 0) continue;
-        const int2 cell = __ldg(g.cells + slot);
-        for (int i = 0; i < cell.y; ++i) f(__ldg(g.sorted + cell.x + i));
-    }
-}
-
-// Sweep 1 of a query at q, one thread: |I| (r_FPFH), |P_normal| (r_normal)
-// and the sum of the P_normal offsets from q, in list order.
-struct Sweep1 {
-    int nf = 0, nn = 0;
-    float sx = 0.f, sy = 0.f, sz = 0.f;
-};
-
-__device__ __forceinline__ Sweep1 sweep1(const GridView& g, const Radii& R, int64_t p, float4 q)
-{
-    Sweep1 r;
-    for_each_candidate(g, p, [&](float4 a) {
-        const float dx = a.x - q.x, dy = a.y - q.y, dz = a.z - q.z;
-        const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-        if (within(a, q, d2, R.rf2, R.rf2d)) {
-            ++r.nf;
-            if (within(a, q, d2, R.rn2, R.rn2d)) {
-                ++r.nn;
-                r.sx += dx;
-                r.sy += dy;
-                r.sz += dz;
-            }
-        }
-    });
-    return r;
-}
-
-// Moments of the P_normal offsets centred on their mean (mx, my, mz), one
-// thread, in list order: s1 (3), then xx xy xz yy yz zz.  With nbr, the
-// r_FPFH neighbours' indices are written from nbr[0] on.
-__device__ __forceinline__ void sweep2(const GridView& g, const Radii& R, int64_t p, float4 q, float mx, float my,
-                                       float mz, float (&mom)[9], int32_t* nbr)
-{
-#pragma unroll
-    for (int i = 0; i < 9; ++i) mom[i] = 0.f;
-    int64_t out = 0;
-    for_each_candidate(g, p, [&](float4 a) {
-        const float dx = a.x - q.x, dy = a.y - q.y, dz = a.z - q.z;
-        const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-        if (!within(a, q, d2, R.rf2, R.rf2d)) return;
-        if (nbr) nbr[out++] = __float_as_int(a.w);
-        if (within(a, q, d2, R.rn2, R.rn2d)) {
-            const float ex = dx - mx, ey = dy - my, ez = dz - mz;
-            mom[0] += ex;
-            mom[1] += ey;
-            mom[2] += ez;
-            mom[3] = fmaf(ex, ex, mom[3]);
-            mom[4] = fmaf(ex, ey, mom[4]);
-            mom[5] = fmaf(ex, ez, mom[5]);
-            mom[6] = fmaf(ey, ey, mom[6]);
-            mom[7] = fmaf(ey, ez, mom[7]);
-            mom[8] = fmaf(ez, ez, mom[8]);
-        }
-    });
-}
-
 // Candidate number t -> position in the sorted point array.
 __device__ __forceinline__ int candidate(int t, int start, int excl)
 {
@@ -200,6 +115,326 @@ __device__ __forceinline__ int candidate(int t, int start, int excl)
     int cs = __shfl_sync(kFull, start, lo);
     int ce = __shfl_sync(kFull, excl, lo);
     return cs + (t - ce);
+}
+
+// Device point count from which the radius searches (normals, the list-free
+// FPFH path) give each query one lane of a warp (LaneQueries); below it one
+// warp takes a query, so that a small cloud still fills the GPU.  Every search
+// kernel applies the same rule, which keeps the list and list-free paths
+// bit-identical.
+constexpr int64_t kThreadQueryMin = 65536;
+
+constexpr int kStep = 4;        // 32-candidate words a warp holds in registers at once
+constexpr int kKeepWords = 32;  // words of P_normal hits kept per query between the two sweeps
+constexpr int kLaneWarps = 4;   // warps per block of the lane-per-query kernels
+
+// Shared memory of one warp of the lane-per-query search.
+struct LaneQueries {
+    float4 neg[32][2];              // the warp's queries negated, each coordinate twice: (x x y y), (z z - -)
+    float4 c[32 * kStep];           // the candidates of the current step
+    unsigned keep[kKeepWords][32];  // r_normal hits of query l in word w
+};
+
+// Candidates of 32 kStep consecutive stencil positions, one per lane and word,
+// the words paired for paired FP32 instructions; lanes past the end hold a
+// point at infinity, which is inside no radius.  Lane 31 holds a word's first
+// candidate, so that the highest set bit of a ballot is the next in list order
+// (one instruction to find).
+struct Words {
+    float2 x[kStep / 2], y[kStep / 2], z[kStep / 2];
+    int idx[kStep];
+
+    __device__ __forceinline__ void load(const GridView& g, int base, int total, int start, int excl, int lane,
+                                         float4* stage)
+    {
+#pragma unroll
+        for (int w = 0; w < kStep; ++w) {
+            const int t = base + 32 * w + 31 - lane;
+            const int pos = candidate(t, start, excl);
+            const float4 a = t < total ? __ldg(g.sorted + pos) : make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+            if (w & 1) {
+                x[w / 2].y = a.x;
+                y[w / 2].y = a.y;
+                z[w / 2].y = a.z;
+            } else {
+                x[w / 2].x = a.x;
+                y[w / 2].x = a.y;
+                z[w / 2].x = a.z;
+            }
+            idx[w] = __float_as_int(a.w);
+            if (stage) stage[32 * w + lane] = a;
+        }
+    }
+};
+
+// The FP64 decision of hit_words for one word: rare, so it is kept out of
+// line (the unrolled tests stay small enough for the instruction cache).
+// Bits 0 and 1: within r_FPFH, within r_normal.
+static __device__ __noinline__ unsigned within_both(float ax, float ay, float az, float qx, float qy, float qz, float d2,
+                                             float rf2, float rn2, double rf2d, double rn2d)
+{
+    const float4 a = make_float4(ax, ay, az, 0.f), q = make_float4(qx, qy, qz, 0.f);
+    if (!(ax < INFINITY)) return 0u;  // no candidate in this lane
+    const bool f = within(a, q, d2, rf2, rf2d);
+    return (f ? 1u : 0u) | (f && within(a, q, d2, rn2, rn2d) ? 2u : 0u);
+}
+
+// Hits of query j among the warp's candidate words: bit l of bf[w] (bn[w]) is
+// set when the candidate of lane l in word w lies within r_FPFH (r_normal).
+// A step in which some distance falls into an FP64 band is decided again.
+template <bool kF, bool kN>
+__device__ __forceinline__ void hit_words(const Words& c, const float4 (&neg)[2], const Radii& R,
+                                          unsigned (&bf)[kStep], unsigned (&bn)[kStep])
+{
+    const float2 qx = make_float2(neg[0].x, neg[0].y), qy = make_float2(neg[0].z, neg[0].w);
+    const float2 qz = make_float2(neg[1].x, neg[1].y);
+    bool band = false;
+    float2 d2[kStep / 2];
+#pragma unroll
+    for (int h = 0; h < kStep / 2; ++h) {
+        const float2 dx = __fadd2_rn(c.x[h], qx), dy = __fadd2_rn(c.y[h], qy), dz = __fadd2_rn(c.z[h], qz);
+        d2[h] = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
+        if (kF) {
+            const float2 e = __fadd2_rn(d2[h], make_float2(-R.rf2, -R.rf2));
+            band |= !(fabsf(e.x) > R.ef);
+            band |= !(fabsf(e.y) > R.ef);
+            bf[2 * h] = __ballot_sync(kFull, e.x < 0.f);
+            bf[2 * h + 1] = __ballot_sync(kFull, e.y < 0.f);
+        }
+        if (kN) {
+            const float2 e = __fadd2_rn(d2[h], make_float2(-R.rn2, -R.rn2));
+            band |= !(fabsf(e.x) > R.en);
+            band |= !(fabsf(e.y) > R.en);
+            bn[2 * h] = __ballot_sync(kFull, e.x < 0.f);
+            bn[2 * h + 1] = __ballot_sync(kFull, e.y < 0.f);
+        }
+    }
+    if (__any_sync(kFull, band)) {
+#pragma unroll
+        for (int w = 0; w < kStep; ++w) {
+            const int h = w / 2;
+            const unsigned in = within_both((w & 1) ? c.x[h].y : c.x[h].x, (w & 1) ? c.y[h].y : c.y[h].x,
+                                            (w & 1) ? c.z[h].y : c.z[h].x, -qx.x, -qy.x, -qz.x,
+                                            (w & 1) ? d2[h].y : d2[h].x, R.rf2, R.rn2, R.rf2d, R.rn2d);
+            if (kF) bf[w] = __ballot_sync(kFull, in & 1u);
+            if (kN) bn[w] = __ballot_sync(kFull, in & 2u);
+        }
+    }
+}
+
+// The lane-per-query kernels take the queries in batches of up to 32 of one
+// cell: positions 0, 32, 64, .. of a cell's run start a batch.  The warp that
+// takes a window of 32 sorted positions takes the batches that start in it, at
+// most 63 queries.  (Batches cut at the windows, whatever the cells, gave 18.4k
+// batches of 16 queries on a 300k-point indoor cloud instead of 14k; whole
+// cells per warp left a tail of dense cells, 0.61 -> 1.03 ms.)
+// Bit l: a batch starts at sorted position p0 + l; (*slot, *end) are that
+// position's cell and the end of its run.
+__device__ __forceinline__ unsigned batch_heads(const GridView& g, int64_t p0, int64_t n_sorted, int lane, int* slot,
+                                                int* end)
+{
+    const int64_t p = p0 + lane;
+    bool head = false;
+    *slot = *end = 0;
+    if (p < n_sorted) {
+        *slot = __ldg(g.sslot + p);
+        const int2 cell = __ldg(g.cells + *slot);
+        *end = cell.x + cell.y;
+        head = (((int)p - cell.x) & 31) == 0;
+    }
+    return __ballot_sync(kFull, head);
+}
+
+// Leave the queries of a batch negated in shared memory, for the whole warp.
+__device__ __forceinline__ void stage_queries(float4 q, int lane, float4 (&neg)[32][2])
+{
+    __syncwarp();
+    neg[lane][0] = make_float4(-q.x, -q.x, -q.y, -q.y);
+    neg[lane][1] = make_float4(-q.z, -q.z, 0.f, 0.f);
+    __syncwarp();
+}
+
+// Calls f(a) for the candidates behind the set bits of the lane's words m, in
+// list order, all lanes together.  A lane moves on to its next word when the
+// current one is used up, so the lanes stay busy until the fullest one ends.
+template <typename F>
+__device__ __forceinline__ void for_each_hit(const unsigned (&words)[kStep], const float4* stage, F&& f)
+{
+    unsigned m[kStep];
+    int left = 0;
+#pragma unroll
+    for (int w = 0; w < kStep; ++w) {
+        m[w] = words[w];
+        left += max(__popc(m[w]), 1);
+    }
+    int at = 0;
+    for (left = __reduce_max_sync(kFull, left); left > 0; --left) {
+        const int bit = 31 - __clz(m[0]);
+        if (m[0]) {
+            f(stage[at + bit]);
+            m[0] ^= 1u << bit;
+        }
+        if (!m[0]) {
+#pragma unroll
+            for (int w = 0; w + 1 < kStep; ++w) m[w] = m[w + 1];
+            m[kStep - 1] = 0u;
+            at += 32;
+        }
+    }
+}
+
+// |I| (r_FPFH), |P_normal| (r_normal) and the centred P_normal moments of the
+// nq <= 32 queries of one batch, one per lane: mom = s1 (3), then xx xy xz yy yz
+// zz of the offsets centred on their mean.  (start, excl, total) is the
+// stencil of their cell (stencil_at).
+//
+// The distance tests run one candidate per lane and one query per step, with
+// the candidates of 4 words held in registers for all queries of the batch; the
+// sums run one query per lane over its hit bits, in list order, the candidate
+// read from shared memory.
+__device__ __forceinline__ void lane_moments(const GridView& g, const Radii& R, int start, int excl, int total, int nq,
+                                             int lane, LaneQueries& sm, float4 q, int* nf_out, int* nn_out,
+                                             float (&mom)[9])
+{
+    stage_queries(q, lane, sm.neg);
+    int nf = 0, nn = 0;
+    float sx = 0.f, sy = 0.f, sz = 0.f;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) mom[i] = 0.f;
+    const bool mine = lane < nq, kept = total <= 32 * kKeepWords;
+    for (int base = 0; base < total; base += 32 * kStep) {
+        Words c;
+        __syncwarp();
+        c.load(g, base, total, start, excl, lane, sm.c);
+        unsigned mf[kStep], mn[kStep];
+#pragma unroll
+        for (int w = 0; w < kStep; ++w) mf[w] = mn[w] = 0u;
+        for (int j = 0; j < nq; ++j) {
+            unsigned bf[kStep], bn[kStep];
+            hit_words<true, true>(c, sm.neg[j], R, bf, bn);
+            if (lane == j) {
+#pragma unroll
+                for (int w = 0; w < kStep; ++w) {
+                    mf[w] = bf[w];
+                    mn[w] = bn[w];
+                }
+            }
+        }
+        const int word0 = kept ? base >> 5 : 0;
+#pragma unroll
+        for (int w = 0; w < kStep; ++w) {
+            nf += __popc(mf[w]);
+            nn += __popc(mn[w]);
+            if (mine) sm.keep[word0 + w][lane] = mn[w];
+        }
+        __syncwarp();
+        for_each_hit(mn, sm.c, [&](float4 e) {
+            sx += e.x - q.x;
+            sy += e.y - q.y;
+            sz += e.z - q.z;
+        });
+    }
+    const float inv = nn > 0 ? 1.0f / (float)nn : 0.0f;
+    const float mx = sx * inv, my = sy * inv, mz = sz * inv;
+    for (int base = 0; base < total; base += 32 * kStep) {
+        const int word0 = kept ? base >> 5 : 0;
+        if (total > 32 * kStep) {  // a single step's candidates are still there
+            Words c;
+            __syncwarp();
+            c.load(g, base, total, start, excl, lane, sm.c);
+            if (!kept) {
+                for (int j = 0; j < nq; ++j) {
+                    unsigned bf[kStep], bn[kStep];
+                    hit_words<false, true>(c, sm.neg[j], R, bf, bn);
+                    if (lane == j) {
+#pragma unroll
+                        for (int w = 0; w < kStep; ++w) sm.keep[w][lane] = bn[w];
+                    }
+                }
+            }
+            __syncwarp();
+        }
+        unsigned mn[kStep];
+#pragma unroll
+        for (int w = 0; w < kStep; ++w) mn[w] = mine ? sm.keep[word0 + w][lane] : 0u;
+        for_each_hit(mn, sm.c, [&](float4 e) {
+            const float dx = e.x - q.x, dy = e.y - q.y, dz = e.z - q.z;
+            const float ex = dx - mx, ey = dy - my, ez = dz - mz;
+            mom[0] += ex;
+            mom[1] += ey;
+            mom[2] += ez;
+            mom[3] = fmaf(ex, ex, mom[3]);
+            mom[4] = fmaf(ex, ey, mom[4]);
+            mom[5] = fmaf(ex, ez, mom[5]);
+            mom[6] = fmaf(ey, ey, mom[6]);
+            mom[7] = fmaf(ey, ez, mom[7]);
+            mom[8] = fmaf(ez, ez, mom[8]);
+        });
+    }
+    *nf_out = nf;
+    *nn_out = nn;
+}
+
+// Every batch of the calling warp's windows: f(q, nq, start, excl, total) with
+// the lane's query (lanes past nq repeat the last one) and its cell's stencil,
+// looked up once per batch, 27 lookups at once.
+template <typename F>
+__device__ __forceinline__ void for_each_batch(const GridView& g, int64_t warp0, int64_t warps, int lane, F&& f)
+{
+    const int64_t n_sorted = *g.n_sorted;
+    for (int64_t p0 = 32 * warp0; p0 < n_sorted; p0 += 32 * warps) {
+        int slot, end;
+        unsigned heads = batch_heads(g, p0, n_sorted, lane, &slot, &end);
+        while (heads) {
+            const int l = __ffs(heads) - 1;
+            heads &= heads - 1u;
+            int cx, cy, cz, start, excl;
+            unpack_cell(__ldg(g.keys + __shfl_sync(kFull, slot, l)), &cx, &cy, &cz);
+            const int total = stencil_at(g, cx, cy, cz, lane, &start, &excl);
+            const int first = (int)p0 + l, nq = min(32, __shfl_sync(kFull, end, l) - first);
+            f(__ldg(g.sorted + first + min(lane, nq - 1)), nq, start, excl, total);
+        }
+    }
+}
+
+// The candidates of the last query a warp searched, kept while the next
+// queries (consecutive in cell order) sit in the same cell: the stencil and its
+// first 32 kStep candidates.
+struct WarpQuery {
+    unsigned long long key = KMX_EMPTY_KEY;
+    int start = 0, excl = 0, total = 0;
+    Words first;
+
+    __device__ __forceinline__ void set(const GridView& g, int64_t p, int lane)
+    {
+        const unsigned long long k = cell_key_at(g, p);
+        if (k == key) return;
+        int x, y, z;
+        unpack_cell(k, &x, &y, &z);
+        total = stencil_at(g, x, y, z, lane, &start, &excl);
+        first.load(g, 0, total, start, excl, lane, nullptr);
+        key = k;
+    }
+
+    // f(words, base) for every 32 kStep candidates
+    template <typename F>
+    __device__ __forceinline__ void for_each(const GridView& g, int lane, F&& f) const
+    {
+        f(first, 0);
+        for (int base = 32 * kStep; base < total; base += 32 * kStep) {
+            Words c;
+            c.load(g, base, total, start, excl, lane, nullptr);
+            f(c, base);
+        }
+    }
+};
+
+// Offset of the lane's candidate in word w from the query (-neg).
+__device__ __forceinline__ float3 offset_of(const Words& c, int w, const float4 (&neg)[2])
+{
+    const int h = w / 2;
+    return make_float3(((w & 1) ? c.x[h].y : c.x[h].x) + neg[0].x, ((w & 1) ? c.y[h].y : c.y[h].x) + neg[0].z,
+                       ((w & 1) ? c.z[h].y : c.z[h].x) + neg[1].x);
 }
 
 __device__ __forceinline__ float warp_sum(float v)
