@@ -275,7 +275,6 @@ __global__ void __launch_bounds__(kThreads) spfh_walk(GridView g, Radii R, const
     __shared__ int hist[kWarps][kStride];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t n_sorted = *g.n_sorted;
-    const float PI = 3.14159265358979f;
     for (int64_t p = (int64_t)blockIdx.x * kWarps + warp; p < n_sorted; p += (int64_t)gridDim.x * kWarps) {
         const float4 q = g.sorted[p];
         const int qi = __float_as_int(q.w);
@@ -289,6 +288,7 @@ __global__ void __launch_bounds__(kThreads) spfh_walk(GridView g, Radii R, const
         if (lane < kStride - 32) hist[warp][32 + lane] = 0;
         __syncwarp();
         const float4 nq = normal4[qi];
+        const bool nq_unit = unit_normal(nq);
         int start, excl;
         const int total = stencil(g, p, lane, &start, &excl);
         int pairs = 0;
@@ -302,13 +302,9 @@ __global__ void __launch_bounds__(kThreads) spfh_walk(GridView g, Radii R, const
                 const float dx = a.x - q.x, dy = a.y - q.y, dz = a.z - q.z;
                 const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
                 if (k != qi && within(a, q, d2, R.rf2, R.rf2d) && (__ldg(&flags[k]) & 1)) {
-                    float f[3];
-                    ok = pair_features(q, nq, a, __ldg(&normal4[k]), f);
-                    if (ok) {
-                        atomicAdd(&hist[warp][feature_bin(f[0], -PI, PI)], 1);
-                        atomicAdd(&hist[warp][kH + feature_bin(f[1], -1.f, 1.f)], 1);
-                        atomicAdd(&hist[warp][2 * kH + feature_bin(f[2], -1.f, 1.f)], 1);
-                    }
+                    const unsigned bins = pair_bins(q, nq, nq_unit, a, __ldg(&normal4[k]));
+                    ok = bins != ~0u;
+                    if (ok) count_bins(hist[warp], bins);
                 }
             }
             pairs += __popc(__ballot_sync(kFull, ok));
