@@ -10,8 +10,8 @@
 //                own slots from offs[q] on)
 //   scan/scatter J in ascending point order
 //   fpfh_kernel  FPFH(q) = SPFH(q) + (1/m) sum_k SPFH(k) / w_k (Eq. A5) over
-//                that stored list, four rows per warp, a lane owning four
-//                bins, compensated summation
+//                that stored list, three rows per warp, a lane owning four
+//                values, compensated summation
 //
 // M[q] is walked once, by the SPFH pass, which gathers every neighbour's
 // point, normal and B anyway; the FPFH pass reads its neighbours and weights
@@ -75,9 +75,8 @@ __global__ void __launch_bounds__(kThreads, 4) spfh_kernel(int64_t n_cap, const 
     // neighbours, most of them from L1 (all points in input order if the grid
     // could not bucket some, which is an error that kmx_sync reports).  Bound
     // by instruction issue: with the bins decided from approximations
-    // (pair_bins) and this order, the whole Faster-PFH chain of a 300k-point
-    // indoor cloud went from 2792 to 2514 us, this kernel's 927 us being a third
-    // of it, with 336 instructions per 32 pairs before
+    // (pair_bins) and this order it went from 927 to 617 us on a 300k-point
+    // indoor cloud (166 neighbours each)
     const bool by_cell = *n_sorted == n;
     for (int64_t p = (int64_t)blockIdx.x * kWarps + warp; p < n; p += (int64_t)gridDim.x * kWarps) {
         const int64_t q = by_cell ? __float_as_int(__ldg(&sorted[p].w)) : p;
@@ -168,67 +167,86 @@ __global__ void __launch_bounds__(kThreads, 4) spfh_kernel(int64_t n_cap, const 
     }
 }
 
-// Four rows per warp: the 8 lanes of group g = lane / 8 take row j of J; lane
-// s = lane % 8 owns bins 4 s .. 4 s + 3 (s = 0 also bin 32) and loads them as
-// one float4 of each neighbour's SPFH row, so the four groups keep four rows
-// in flight per step.  The neighbours and weights come from the list
-// spfh_kernel stored (coalesced, eight entries per group and step, passed
-// between the group's lanes by shuffles).  Every bin adds its neighbours'
-// values in list order with the compensated product-sum the list-free path
-// uses (the same bits; the four bins of a lane go through it in pairs,
-// kahan_add_prod2).
-__global__ void __launch_bounds__(kThreads, 6) fpfh_kernel(int64_t n_cap, const int32_t* __restrict__ valid,
-                                                           const int64_t* __restrict__ n_valid,
+// Three rows per warp: the 9 lanes of group g = lane / 9 take one row of J
+// (lanes 27 .. 31 idle); lane s of a group owns the four values at 4 s of the
+// 36-float row (the last holds bin 32 and the padding), one float4 of each
+// neighbour's SPFH row.  (Eight lanes and four rows per warp left bin 32 to one
+// lane, in a branch of its own: 13 instructions per neighbour instead of 6.)
+// The neighbours and weights come from the list spfh_kernel stored (coalesced,
+// nine entries per group and step, passed between the group's lanes by
+// shuffles).  Every bin adds its neighbours' values in list order with the
+// compensated product-sum the list-free path uses (the same bits; the four
+// values of a lane go through it in pairs, kahan_add_prod2).
+constexpr int kRowLanes = kStride / 4;  // 9
+constexpr int kRowsPerWarp = 32 / kRowLanes;
+
+__global__ void __launch_bounds__(kThreads, 6) fpfh_kernel(int64_t n_cap, const int64_t* d_n,
+                                                           const float4* __restrict__ sorted,
+                                                           const int64_t* __restrict__ n_sorted,
+                                                           const uint8_t* __restrict__ flags,
+                                                           const int64_t* __restrict__ jpos,
                                                            const int64_t* __restrict__ offs,
                                                            const int2* __restrict__ wlist,
                                                            const int32_t* __restrict__ wcnt,
                                                            const float* __restrict__ spfh, float* __restrict__ desc)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 3, s = lane & 7;
-    const int lead = lane & ~7;  // lane 0 of the group
-    const int64_t nv = min(*n_valid, n_cap);
-    const int64_t warps = (int64_t)gridDim.x * kWarps;
-    for (int64_t w4 = (int64_t)blockIdx.x * kWarps + warp; w4 * 4 < nv; w4 += warps) {
-        const int64_t j = w4 * 4 + g;
-        const bool active = j < nv;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane / kRowLanes, s = lane - g * kRowLanes;
+    const int lead = g * kRowLanes;
+    const int64_t n = kmx_count(d_n, n_cap);
+    const bool by_cell = *n_sorted == n;  // as in spfh_kernel
+    const int64_t step = (int64_t)gridDim.x * kWarps * kRowsPerWarp;
+    for (int64_t p0 = ((int64_t)blockIdx.x * kWarps + warp) * kRowsPerWarp; p0 < n; p0 += step) {
+        const int64_t p = p0 + g;
         int q = 0, m = 0;
         int64_t b = 0;
+        bool active = g < kRowsPerWarp && p < n;
         if (active) {
-            q = valid[j];
-            b = offs[q];
-            m = wcnt[q];
+            q = by_cell ? __float_as_int(__ldg(&sorted[p].w)) : (int)p;
+            active = (flags[q] & 2) != 0;
+            if (active) {
+                b = offs[q];
+                m = wcnt[q];
+            }
         }
-        // bins 4 s .. 4 s + 3 as two pairs of sums (negated compensations)
+        // values 4 s .. 4 s + 3 as two pairs of sums (negated compensations)
         float2 acc01 = make_float2(0.f, 0.f), acc23 = make_float2(0.f, 0.f);
         float2 nc01 = make_float2(0.f, 0.f), nc23 = make_float2(0.f, 0.f);
-        float acc32 = 0.f, comp32 = 0.f;
-        for (int c = 0; __any_sync(kFull, c < m); c += 8) {
-            const int cnt = min(max(m - c, 0), 8);  // this group's entries in the chunk
+        for (int c = 0; __any_sync(kFull, c < m); c += kRowLanes) {
+            const int cnt = min(max(m - c, 0), kRowLanes);  // this group's entries in the chunk
             const int2 ent = s < cnt ? __ldg(&wlist[b + c + s]) : make_int2(0, 0);
-            const int steps = __reduce_max_sync(kFull, (unsigned)cnt);
-#pragma unroll 4
-            for (int i = 0; i < steps; ++i) {
-                const int k = __shfl_sync(kFull, ent.x, lead + i);
-                const float we = __int_as_float(__shfl_sync(kFull, ent.y, lead + i));
-                if (i < cnt) {
-                    const float* r = spfh + (int64_t)k * kStride;
-                    const float4 v = __ldg(reinterpret_cast<const float4*>(r) + s);
+            // a row without entries takes part in whole steps too: its sums are
+            // not used
+            if (__all_sync(kFull, cnt == kRowLanes || m == 0)) {
+#pragma unroll
+                for (int i = 0; i < kRowLanes; ++i) {
+                    const int k = __shfl_sync(kFull, ent.x, lead + i);
+                    const float we = __int_as_float(__shfl_sync(kFull, ent.y, lead + i));
+                    const float4 v = __ldg(reinterpret_cast<const float4*>(spfh + (int64_t)k * kStride) + s);
                     const float2 we2 = make_float2(we, we);
                     kahan_add_prod2(acc01, nc01, make_float2(v.x, v.y), we2);
                     kahan_add_prod2(acc23, nc23, make_float2(v.z, v.w), we2);
-                    if (s == 0) kahan_add_prod(acc32, comp32, __ldg(&r[32]), we);
+                }
+            } else {
+                const int steps = __reduce_max_sync(kFull, (unsigned)cnt);
+                for (int i = 0; i < steps; ++i) {
+                    const int k = __shfl_sync(kFull, ent.x, lead + i);
+                    const float we = __int_as_float(__shfl_sync(kFull, ent.y, lead + i));
+                    if (i < cnt) {
+                        const float4 v = __ldg(reinterpret_cast<const float4*>(spfh + (int64_t)k * kStride) + s);
+                        const float2 we2 = make_float2(we, we);
+                        kahan_add_prod2(acc01, nc01, make_float2(v.x, v.y), we2);
+                        kahan_add_prod2(acc23, nc23, make_float2(v.z, v.w), we2);
+                    }
                 }
             }
         }
         if (active) {
-            const float* rq = spfh + (int64_t)q * kStride;
             const float invm = m > 0 ? 1.0f / (float)m : 0.f;
-            float* out = desc + j * kStride;
-            const float4 rv = reinterpret_cast<const float4*>(rq)[s];
-            reinterpret_cast<float4*>(out)[s] = make_float4(fmaf(acc01.x, invm, rv.x), fmaf(acc01.y, invm, rv.y),
-                                                            fmaf(acc23.x, invm, rv.z), fmaf(acc23.y, invm, rv.w));
-            if (s == 0)
-                reinterpret_cast<float4*>(out)[8] = make_float4(fmaf(acc32, invm, rq[32]), 0.f, 0.f, 0.f);
+            const float4 rv = __ldg(reinterpret_cast<const float4*>(spfh + (int64_t)q * kStride) + s);
+            reinterpret_cast<float4*>(desc + jpos[q] * kStride)[s] =
+                m > 0 ? make_float4(fmaf(acc01.x, invm, rv.x), fmaf(acc01.y, invm, rv.y), fmaf(acc23.x, invm, rv.z),
+                                    fmaf(acc23.y, invm, rv.w))
+                      : rv;
         }
     }
 }
@@ -256,7 +274,7 @@ cudaError_t kmx_fasterpfh_launch(kmx_ctx* ctx, const kmx_grid* g, const kmx_para
     // about the same, so every resident block takes an equal share
     unsigned nbs = 0, nbf = 0;
     if ((e = kmx_wave_blocks(spfh_kernel, kThreads, 0, n, kWarps, ctx->sm_count, &nbs))) return e;
-    if ((e = kmx_wave_blocks(fpfh_kernel, kThreads, 0, n, 4 * kWarps, ctx->sm_count, &nbf))) return e;
+    if ((e = kmx_wave_blocks(fpfh_kernel, kThreads, 0, n, kRowsPerWarp * kWarps, ctx->sm_count, &nbf))) return e;
     // spfh_kernel writes the J flag of every point below the count; the scan
     // reads no other entry
     KMX_COUNT_LAUNCH();
@@ -268,6 +286,7 @@ cudaError_t kmx_fasterpfh_launch(kmx_ctx* ctx, const kmx_grid* g, const kmx_para
     scatter_valid<<<kmx_stride_blocks(n, kThreads, ctx->sm_count), kThreads, 0, st>>>(n, g->d_n, s.jflag, s.jpos,
                                                                                        valid, n_valid);
     KMX_COUNT_LAUNCH();
-    fpfh_kernel<<<nbf, kThreads, 0, st>>>(n, valid, n_valid, offs, s.wlist, s.wcnt, sp, desc);
+    fpfh_kernel<<<nbf, kThreads, 0, st>>>(n, g->d_n, g->sorted, g->d_n_sorted, flags, s.jpos, offs, s.wlist, s.wcnt, sp,
+                                          desc);
     return cudaGetLastError();
 }
