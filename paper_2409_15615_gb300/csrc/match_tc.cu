@@ -39,14 +39,13 @@
 //             its own centre and radius, then row by row, with margins for
 //             FP32 rounding).  The tiles that pass form the row tile's list,
 //             cut into work items of 32 tiles.
-//   collect   persistent CTAs, each taking every gridDim-th work item: per
+//   collect   persistent CTAs (two per SM), each taking every gridDim-th work item: per
 //             column tile of the item the CTA writes its row tile re-centred
 //             on the column tile's centre as the A operand
 //             [x - c_C, sqrt(c') |x - c_C|, -1/2, -1/2] while earlier tiles'
 //             products run, one thread issues tcgen05.mma (kind::f16, BF16,
-//             M = N = 128, three K steps of 16) into one of four TMEM
-//             accumulators, and two warpgroups of four warps read them
-//             with tcgen05.ld (alternate tiles, two tiles in flight).  The
+//             M = N = 128, three K steps of 16) into one of two TMEM
+//             accumulators, and four warps read them with tcgen05.ld.  The
 //             accumulator holds M = a.b + c' |a| |b| - |b|^2 / 2
 //             (approximately), so L = |a|^2 - 2 M - e is a certified lower
 //             bound of the exact d^2, and L + 4.1 c' |a| |b| + 2 e an upper
@@ -111,13 +110,14 @@ constexpr int kHdrCenter = kHdrBeta + kTN * 4;
 constexpr int kHdrBmax = kHdrCenter + kCenterStride * 4;
 constexpr int kHdrGBeta = kHdrBmax + 16;
 constexpr int kColBytes = kHdrGBeta + (kTN / 8) * 4;  // 13024, a multiple of 16
-constexpr int kStages = 6;                    // column-tile ring
-constexpr int kThreads = 512;                 // 16 warps (roles in tc_collect)
-constexpr int kTmemCols = 512;                // four 128-column FP32 accumulators
+constexpr int kStages = 4;                    // column-tile ring
+constexpr int kThreads = 320;                 // 10 warps (roles in tc_collect)
+constexpr int kCtasPerSm = 2;                 // of tc_collect
+constexpr int kTmemCols = 256;                // two 128-column FP32 accumulators per CTA
 constexpr int kCandCap = 512;                 // candidate list per row
-constexpr int kItemTiles = 32;                // column tiles per work item
+constexpr int kItemTiles = 32;                // column tiles per work item (a power of two)
 constexpr int kPlanRec = 32;                  // columns of the nearest tile recorded per row in the plan
-constexpr int kCandBuf = 16;                  // candidates buffered per row and epilogue warpgroup in the collect kernel
+constexpr int kCandBuf = 16;                  // candidates buffered per row in the collect kernel
 constexpr float kC = 0.008f;                  // c' of the bounds
 constexpr float kSqrtC = 0.08944271909999159f;
 constexpr float kUpper = 4.1f * kC;
@@ -183,39 +183,27 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar)
                  : "memory");
 }
 
-// 64 consecutive FP32 columns of this thread's TMEM lane: two loads in
-// flight, one wait.
-__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float* v)
+// 32 consecutive FP32 columns of this thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v)
 {
-    uint32_t r[64];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        uint32_t* q = r + 32 * h;
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-            "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-            : "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7]),
-              "=r"(q[8]), "=r"(q[9]), "=r"(q[10]), "=r"(q[11]), "=r"(q[12]), "=r"(q[13]), "=r"(q[14]), "=r"(q[15]),
-              "=r"(q[16]), "=r"(q[17]), "=r"(q[18]), "=r"(q[19]), "=r"(q[20]), "=r"(q[21]), "=r"(q[22]), "=r"(q[23]),
-              "=r"(q[24]), "=r"(q[25]), "=r"(q[26]), "=r"(q[27]), "=r"(q[28]), "=r"(q[29]), "=r"(q[30]), "=r"(q[31])
-            : "r"(taddr + 32 * h));
-    }
+    uint32_t q[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+        "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7]),
+          "=r"(q[8]), "=r"(q[9]), "=r"(q[10]), "=r"(q[11]), "=r"(q[12]), "=r"(q[13]), "=r"(q[14]), "=r"(q[15]),
+          "=r"(q[16]), "=r"(q[17]), "=r"(q[18]), "=r"(q[19]), "=r"(q[20]), "=r"(q[21]), "=r"(q[22]), "=r"(q[23]),
+          "=r"(q[24]), "=r"(q[25]), "=r"(q[26]), "=r"(q[27]), "=r"(q[28]), "=r"(q[29]), "=r"(q[30]), "=r"(q[31])
+        : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(q[i]);
 }
 
 __device__ __forceinline__ float fmax3(float a, float b, float c)
 {
     float d;
     asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-
-__device__ __forceinline__ float fmin3(float a, float b, float c)
-{
-    float d;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
     return d;
 }
 
@@ -1015,6 +1003,13 @@ __device__ __forceinline__ bool tile_may_hold(float dist, float rad, float u2)
     return !(g > 0.f && g * g * (1.f - kTolD) > u2);
 }
 
+// A work item: a row tile, the first of its list's column tiles (a multiple of
+// kItemTiles) and, in the low bits, how many tiles less one.
+__device__ __forceinline__ int2 pack_item(int rt, int first, int total)
+{
+    return make_int2(rt, first | (min(kItemTiles, total - first) - 1));
+}
+
 // One CTA of 128 threads (thread = row) per row tile rt of X, with cenX and
 // cenY the centres and squared radii of both clouds' tiles (tc_pack).
 //   1. the column tile cs with the centre nearest to the row tile's centre
@@ -1312,7 +1307,7 @@ __device__ __forceinline__ void plan_tile(const float* __restrict__ X, const int
         const int nit = (total + kItemTiles - 1) / kItemTiles;
         if (nit > 0) {
             const int b = atomicAdd(n_items, nit);
-            for (int i = 0; i < nit; ++i) items[b + i] = make_int2((int)rt, i * kItemTiles);
+            for (int i = 0; i < nit; ++i) items[b + i] = pack_item((int)rt, i * kItemTiles, total);
         }
     }
 }
@@ -1365,12 +1360,8 @@ __global__ void __launch_bounds__(kTM) tc_plan(PlanDir a, PlanDir b, int* __rest
 // tensor-core candidate collection
 // ---------------------------------------------------------------------------
 
-constexpr int kAStages = 6;   // re-centred row tiles in flight
-constexpr int kAccBufs = 4;   // TMEM accumulators (4 x 128 columns: the whole TMEM)
-// Tile t goes to epilogue warpgroup t % 2; with even ring sizes every phase
-// of a barrier of the A ring or of the accumulators gets its arrivals from
-// the same warpgroup.
-static_assert(kAStages % 2 == 0 && kAccBufs % 2 == 0, "rings alternate between the two epilogue warpgroups");
+constexpr int kAStages = 3;   // re-centred row tiles in flight
+constexpr int kAccBufs = 2;   // TMEM accumulators (2 x 128 columns: half of the TMEM)
 
 struct TcShared {
     uint8_t a[kAStages][kOpBytesA];
@@ -1378,54 +1369,54 @@ struct TcShared {
     // per row and A stage: |a|^2 - e, the factor c' |a| of the upper bounds, 2 e
     float4 rowc[kAStages][kTM];
     float gb[kAStages][kTN / 8];  // the column tile's largest |b| per group of 8
-    float2 ul[kTM][2];            // latest (U1, U2) of every row from each epilogue warpgroup
-    // candidates of the current item per (warpgroup, row), appended to the row's
-    // global list when full and at the item's end (stride 17: no bank conflicts)
-    int32_t cbuf[2][kTM][kCandBuf + 1];
+    // candidates of the current item per row, appended to the row's global
+    // list when full and at the item's end (stride 17: no bank conflicts)
+    int32_t cbuf[kTM][kCandBuf + 1];
     uint64_t full_b[kStages], empty_b[kStages];
     uint64_t full_a[kAStages], empty_a[kAStages];
     uint64_t acc_full[kAccBufs], acc_empty[kAccBufs];
     uint32_t tmem;
     int failed;
 };
+// kCtasPerSm CTAs fit an SM's shared memory (1 KB of it is each CTA's own) and
+// its TMEM; a further one does not fit the shared memory, so none ever waits
+// in tcgen05.alloc.
+static_assert(kCtasPerSm * (sizeof(TcShared) + 2048) <= 228 * 1024 && kCtasPerSm * kTmemCols <= 512 &&
+                  (kCtasPerSm + 1) * sizeof(TcShared) > 228 * 1024,
+              "tc_collect: CTAs per SM");
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-// Epilogue warps only (warps 8..15).
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-
-// Persistent CTAs; CTA b takes the work items b, b + gridDim.x, ... (an item
-// is up to kItemTiles column tiles of one row tile's list).  Warp roles (16
-// warps), each running its own loop over the CTA's sequence of column tiles
-// and handing tiles on through mbarriers, so that copying, re-centring,
-// tensor-core products and the epilogue of different tiles overlap:
-//   warp 1 (lane 0)   producer: bulk-copies column tiles into a 4-stage ring;
-//   warps 4..7        re-centring: thread = row; the row re-centred on the
+// Persistent CTAs, two per SM; CTA b takes the work items b, b + gridDim.x, ...
+// (an item is up to kItemTiles column tiles of one row tile's list).  Warp
+// roles (10 warps), each running its own loop over the CTA's sequence of
+// column tiles and handing tiles on through mbarriers, so that copying,
+// re-centring, tensor-core products and the epilogue of different tiles
+// overlap:
+//   warps 0..3        re-centring: thread = row; the row re-centred on the
 //                     column tile's centre as the A operand (3-stage ring),
 //                     and the row's constants of the bounds;
-//   warp 0 (lane 0)   issues tcgen05.mma (M = N = 128, three K steps) into one
-//                     of four TMEM accumulators and commits to the barriers
+//   warps 4..7        epilogue: thread = row; warp w reads TMEM lanes
+//                     32 (w & 3) .. + 31, all 128 columns of the tile's
+//                     accumulator in four quarters of 32;
+//   warp 8 (lane 0)   issues tcgen05.mma (M = N = 128, three K steps) into one
+//                     of two TMEM accumulators and commits to the barriers
 //                     that free the accumulator's reader, the A stage and the
 //                     B stage;
-//   warps 8..15       epilogue, two warpgroups: warps 8..11 take the tiles
-//                     t with t % 2 == 0, warps 12..15 the others; warp w reads
-//                     TMEM lanes 32 (w & 3) .. + 31, all 128 columns of the
-//                     tile's accumulator in two halves of 64.
-// The two epilogue threads of a row (one per warpgroup) keep their own upper
-// bounds over their own tiles' columns and publish them after every tile;
-// each combines its own with the other's latest published pair (their column
-// sets are disjoint, so any snapshot is a valid bound).  Both start an item from the row's bound U
-// counted as two columns at U (the two best columns of the plan's tile,
-// which no item holds); at an item boundary the epilogue warps meet on a
-// named barrier, so that no thread reads a bound of the previous item's row.
-__global__ void __launch_bounds__(kThreads, 1) tc_collect(const float* __restrict__ X,
+//   warp 9 (lane 0)   producer: bulk-copies column tiles into a 4-stage ring.
+// What bounds it: a tile's way through the four roles, each a serial chain of
+// barrier waits, shared-memory and TMEM loads; no unit is busy (tensor cores
+// about a fifth of the time).  Two CTAs give every SM two such chains: the
+// match of 302548 x 287858 indoor descriptors, with one CTA of 16 warps per SM
+// (two epilogue warpgroups) before, went from 6.06 to 5.45 ms.  The epilogue
+// reads 32 columns at a time because 64 spill at 96 registers (6.0 ms).
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) tc_collect(const float* __restrict__ X,
                                                          const int32_t* __restrict__ permX, int64_t nx_cap,
                                                          const int64_t* d_nx, const uint8_t* __restrict__ packY,
                                                          const int32_t* __restrict__ need, int64_t need_stride,
-                                                         const int32_t* __restrict__ nneed,
                                                          const int2* __restrict__ items, const int* __restrict__ n_items,
                                                          float* __restrict__ ub, int32_t* __restrict__ cand,
                                                          int32_t* __restrict__ cnt, unsigned int* err)
@@ -1437,12 +1428,13 @@ __global__ void __launch_bounds__(kThreads, 1) tc_collect(const float* __restric
     const int nit = *n_items;
     if ((int)blockIdx.x >= nit) return;
     const int stride = (int)gridDim.x;
-    auto item_tiles = [&](int it, const int32_t*& tl, int64_t& rt) -> int {
-        const int2 item = items[it];
+    auto item_tiles = [&](int2 item, const int32_t*& tl, int64_t& rt) -> int {
         rt = item.x;
-        tl = need + (int64_t)item.x * need_stride + item.y;
-        return min(kItemTiles, nneed[item.x] - item.y);
+        tl = need + (int64_t)item.x * need_stride + (item.y & ~(kItemTiles - 1));
+        return (item.y & (kItemTiles - 1)) + 1;
     };
+    // the next item is read an item ahead, so that no role waits for it
+    auto item_at = [&](int it) -> int2 { return it < nit ? __ldg(items + it) : make_int2(0, 0); };
 
     if (tid == 0) {
         for (int st = 0; st < kStages; ++st) {
@@ -1451,16 +1443,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc_collect(const float* __restric
         }
         for (int st = 0; st < kAStages; ++st) {
             mbar_init(&S.full_a[st], 4);           // re-centring warps
-            mbar_init(&S.empty_a[st], 1 + 4);      // MMA commit + the 4 warps of the tile's epilogue warpgroup
+            mbar_init(&S.empty_a[st], 1 + 4);      // MMA commit + the 4 epilogue warps
         }
         for (int k = 0; k < kAccBufs; ++k) {
             mbar_init(&S.acc_full[k], 1);          // MMA commit
-            mbar_init(&S.acc_empty[k], 4);         // the 4 warps of the tile's epilogue warpgroup
+            mbar_init(&S.acc_empty[k], 4);         // the 4 epilogue warps
         }
         mbar_fence_init();
         S.failed = 0;
     }
-    if (warp == 0) tmem_alloc(&S.tmem, kTmemCols);
+    if (warp == 8) tmem_alloc(&S.tmem, kTmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1468,14 +1460,16 @@ __global__ void __launch_bounds__(kThreads, 1) tc_collect(const float* __restric
     volatile int* failed = &S.failed;
     int issued_b = 0, issued_mma = 0;
 
-    if (warp == 1) {
+    if (warp == 9) {
         // ---- producer
         if (lane == 0) {
             int t = 0;
+            int2 item = item_at(blockIdx.x);
             for (int it = blockIdx.x; it < nit && !*failed; it += stride) {
                 const int32_t* tl;
                 int64_t rt;
-                const int nt = item_tiles(it, tl, rt);
+                const int nt = item_tiles(item, tl, rt);
+                item = item_at(it + stride);
                 for (int k = 0; k < nt; ++k, ++t) {
                     const int st = t % kStages;
                     if (t >= kStages && !mbar_wait(&S.empty_b[st], ((t / kStages) - 1) & 1)) {
@@ -1488,15 +1482,17 @@ __global__ void __launch_bounds__(kThreads, 1) tc_collect(const float* __restric
                 }
             }
         }
-    } else if (warp == 0) {
+    } else if (warp == 8) {
         // ---- tensor-core products
         if (lane == 0) {
             const uint32_t idesc = idesc_bf16(kTM, kTN);
             int t = 0;
+            int2 item = item_at(blockIdx.x);
             for (int it = blockIdx.x; it < nit && !*failed; it += stride) {
                 const int32_t* tl;
                 int64_t rt;
-                const int nt = item_tiles(it, tl, rt);
+                const int nt = item_tiles(item, tl, rt);
+                item = item_at(it + stride);
                 for (int k = 0; k < nt; ++k, ++t) {
                     const int st = t % kStages, sa = t % kAStages, ab = t % kAccBufs;
                     bool ok = mbar_wait(&S.full_b[st], (t / kStages) & 1) &&
@@ -1523,24 +1519,34 @@ __global__ void __launch_bounds__(kThreads, 1) tc_collect(const float* __restric
                 }
             }
         }
-    } else if (warp >= 4 && warp < 8) {
+    } else if (warp < 4) {
         // ---- re-centring: thread = row
-        const int rrow = tid - 128;
+        const int rrow = tid;
         int64_t cur = -1;
         float x[KMX_DESC_DIM];
         int t = 0;
         bool dead = false;
+        int2 item = item_at(blockIdx.x);
         for (int it = blockIdx.x; it < nit && !dead; it += stride) {
             const int32_t* tl;
             int64_t rt;
-            const int nt = item_tiles(it, tl, rt);
+            const int nt = item_tiles(item, tl, rt);
+            item = item_at(it + stride);
             if (rt != cur) {
                 cur = rt;
                 const int64_t xrow = rt * kTM + rrow;
                 const bool xvalid = xrow < rows;
-                const float* xr = xvalid ? X + (int64_t)permX[xrow] * KMX_DESC_STRIDE : nullptr;
+                const float4* x4 =
+                    reinterpret_cast<const float4*>(X + (xvalid ? (int64_t)permX[xrow] * KMX_DESC_STRIDE : 0));
 #pragma unroll
-                for (int h = 0; h < KMX_DESC_DIM; ++h) x[h] = xvalid ? __ldg(xr + h) : 0.f;
+                for (int q = 0; q < 8; ++q) {
+                    const float4 xv = xvalid ? __ldg(x4 + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    x[4 * q] = xv.x;
+                    x[4 * q + 1] = xv.y;
+                    x[4 * q + 2] = xv.z;
+                    x[4 * q + 3] = xv.w;
+                }
+                x[32] = xvalid ? __ldg(reinterpret_cast<const float*>(x4) + 32) : 0.f;
             }
             for (int k = 0; k < nt; ++k, ++t) {
                 const int st = t % kStages, sa = t % kAStages;
@@ -1554,32 +1560,33 @@ __global__ void __launch_bounds__(kThreads, 1) tc_collect(const float* __restric
                 }
                 const uint8_t* bt = S.b[st];
                 const float4* cen4 = reinterpret_cast<const float4*>(bt + kHdrCenter);
-                float v[kK];
+                uint8_t* arow = S.a[sa] + (rrow / 8) * kGroupStride + (rrow % 8) * 16;
                 // paired FP32 operations (the same per-lane rounding); |a|^2
                 // as two interleaved partial sums
                 float2 q2 = make_float2(0.f, 0.f);
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const float4 cv = cen4[c];
+                for (int c = 0; c < 4; ++c) {  // eight values: one 16-byte row of a core matrix
+                    const float4 ca = cen4[2 * c], cb = cen4[2 * c + 1];
                     // x + (-c) is exactly x - c
-                    const float2 d0 = __fadd2_rn(make_float2(x[4 * c + 0], x[4 * c + 1]), make_float2(-cv.x, -cv.y));
-                    const float2 d1 = __fadd2_rn(make_float2(x[4 * c + 2], x[4 * c + 3]), make_float2(-cv.z, -cv.w));
-                    v[4 * c + 0] = d0.x;
-                    v[4 * c + 1] = d0.y;
-                    v[4 * c + 2] = d1.x;
-                    v[4 * c + 3] = d1.y;
+                    const float2 d0 = __fadd2_rn(make_float2(x[8 * c + 0], x[8 * c + 1]), make_float2(-ca.x, -ca.y));
+                    const float2 d1 = __fadd2_rn(make_float2(x[8 * c + 2], x[8 * c + 3]), make_float2(-ca.z, -ca.w));
+                    const float2 d2 = __fadd2_rn(make_float2(x[8 * c + 4], x[8 * c + 5]), make_float2(-cb.x, -cb.y));
+                    const float2 d3 = __fadd2_rn(make_float2(x[8 * c + 6], x[8 * c + 7]), make_float2(-cb.z, -cb.w));
                     q2 = __ffma2_rn(d0, d0, q2);
                     q2 = __ffma2_rn(d1, d1, q2);
+                    q2 = __ffma2_rn(d2, d2, q2);
+                    q2 = __ffma2_rn(d3, d3, q2);
+                    *reinterpret_cast<uint4*>(arow + c * kCoreStride) =
+                        make_uint4(pack_bf16x2(d0.x, d0.y), pack_bf16x2(d1.x, d1.y), pack_bf16x2(d2.x, d2.y),
+                                   pack_bf16x2(d3.x, d3.y));
                 }
-                v[32] = x[32] - reinterpret_cast<const float*>(bt + kHdrCenter)[32];
-                const float p2 = fmaf(v[32], v[32], q2.x + q2.y);
+                const float v32 = x[32] - reinterpret_cast<const float*>(bt + kHdrCenter)[32];
+                const float p2 = fmaf(v32, v32, q2.x + q2.y);
                 const float al = sqrtf(p2);
-                v[KMX_DESC_DIM] = kSqrtC * al;
-                v[KMX_DESC_DIM + 1] = -0.5f;
-                v[KMX_DESC_DIM + 2] = -0.5f;
-#pragma unroll
-                for (int h = KMX_DESC_DIM + 3; h < kK; ++h) v[h] = 0.f;
-                store_operand_row(S.a[sa], rrow, v);
+                *reinterpret_cast<uint4*>(arow + 4 * kCoreStride) =
+                    make_uint4(pack_bf16x2(v32, kSqrtC * al), pack_bf16x2(-0.5f, -0.5f), 0u, 0u);
+                // the last eight K slots stay zero: written in each stage's first use
+                if (t < kAStages) *reinterpret_cast<uint4*>(arow + 5 * kCoreStride) = make_uint4(0u, 0u, 0u, 0u);
                 const float bmax2 = reinterpret_cast<const float*>(bt + kHdrBmax)[0];
                 const float ef = kEfp * (p2 + bmax2);
                 S.rowc[sa][rrow] = make_float4(p2 - ef, kUpper * al, 2.f * ef, 0.f);
@@ -1592,11 +1599,11 @@ __global__ void __launch_bounds__(kThreads, 1) tc_collect(const float* __restric
                 }
             }
         }
-    } else if (warp >= 8) {
+    } else {
         // ---- epilogue
-        const int quarter = warp & 3, wg = (warp - 8) >> 2;  // warpgroup wg takes the tiles t with t % 2 == wg
+        const int quarter = warp & 3;
         const int r = quarter * 32 + lane;
-        int32_t* cbuf = S.cbuf[wg][r];
+        int32_t* cbuf = S.cbuf[r];
         int nbuf = 0;
         // one atomic per flush reserves the places in the row's global list
         auto flush_cands = [&](int64_t row, int nb) {
@@ -1604,75 +1611,69 @@ __global__ void __launch_bounds__(kThreads, 1) tc_collect(const float* __restric
             for (int i = 0; i < nb; ++i)
                 if (pos + i < kCandCap) cand[row * kCandCap + pos + i] = cbuf[i];
         };
+        // the row's latest bound; rows past the end have none
+        auto bound_at = [&](int rt) -> float {
+            const int64_t row = (int64_t)rt * kTM + r;
+            return row < rows ? __ldcg(ub + row) : FLT_MAX;
+        };
         int t = 0;
         bool dead = false;
-        // every epilogue warp runs every item (after a failure without
-        // waiting or working), so that all meet on each named barrier
-        for (int it = blockIdx.x; it < nit; it += stride) {
+        int2 item = item_at(blockIdx.x);
+        float Unext = bound_at(item.x);
+        for (int it = blockIdx.x; it < nit && !dead; it += stride) {
             const int32_t* tl;
             int64_t rt;
-            const int nt = item_tiles(it, tl, rt);
+            const int nt = item_tiles(item, tl, rt);
+            item = item_at(it + stride);
             const int64_t row = rt * kTM + r;
             const bool row_valid = row < rows;
-            float U1 = row_valid ? __ldcg(ub + row) : FLT_MAX, U2 = U1;
-            epi_sync();  // the previous item's bounds are no longer read
-            *reinterpret_cast<volatile unsigned long long*>(&S.ul[r][wg]) =
-                (unsigned long long)__float_as_uint(U1) | ((unsigned long long)__float_as_uint(U2) << 32);
-            epi_sync();
+            // the row's bound U counts as two columns at U (the two best
+            // columns of the plan's tile, which no item holds)
+            float U1 = Unext, U2 = Unext;
             for (int k = 0; k < nt; ++k, ++t) {
-                if ((t & 1) != wg) continue;  // the other warpgroup's tile
                 const int sa = t % kAStages, ab = t % kAccBufs;
-                if (dead) continue;
+                const int tile = tl[k];
+                if (k + 1 == nt) Unext = bound_at(item.x);
                 bool ok = !*failed;
                 if (ok) ok = mbar_wait(&S.acc_full[ab], (t / kAccBufs) & 1);
-                // the A stage (row constants) cannot be refilled before this
-                // warpgroup's arrival on empty_a, so its phase t / kAStages is
+                // the A stage (row constants) cannot be refilled before these
+                // warps' arrival on empty_a, so its phase t / kAStages is
                 // the current one: the wait only acquires the re-centring writes
                 if (ok) ok = mbar_wait(&S.full_a[sa], (t / kAStages) & 1);
                 if (!__all_sync(0xffffffffu, ok)) {
                     if (lane == 0) *failed = 1;
                     dead = true;
-                    continue;
+                    break;
                 }
                 tc_fence_after();
                 const float4 rc = S.rowc[sa][r];
                 const float rb = rc.x, ua = rc.y, ue = rc.z;
-                // one 64-bit load: the pair is never seen half written
-                const unsigned long long ou = *reinterpret_cast<volatile unsigned long long*>(&S.ul[r][wg ^ 1]);
-                const float2 other =
-                    make_float2(__uint_as_float((uint32_t)ou), __uint_as_float((uint32_t)(ou >> 32)));
                 const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ab * kTN);
 #pragma unroll 1
-                for (int h = 0; h < 2; ++h) {  // the two 64-column halves of the tile
-                    float v[64];
-                    tmem_ld64(tbase + (uint32_t)(h * 64), v);
-                    if (h == 1) {
+                for (int h = 0; h < 4; ++h) {  // the four 32-column quarters of the tile
+                    float v[32];
+                    tmem_ld32(tbase + (uint32_t)(h * 32), v);
+                    if (h == 3) {
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&S.acc_empty[ab]);  // the accumulator is read
                     }
-                    const float* gbeta = S.gb[sa] + h * 8;
-                    const int64_t col0 = (int64_t)tl[k] * kTN + h * 64;
-                    // the second-smallest upper bound over both warpgroups' columns
-                    const float Ush = fminf(fmaxf(U1, other.x), U1 <= other.x ? U2 : other.y);
-                    float Lm[8];
+                    const float* gbeta = S.gb[sa] + h * 4;
+                    const int col0 = tile * kTN + h * 32;
+                    float Mm[4];
 #pragma unroll
-                    for (int g = 0; g < 8; ++g) {
+                    for (int g = 0; g < 4; ++g) {
                         const float* vg = v + 8 * g;
-                        const float m =
-                            fmax3(fmax3(vg[0], vg[1], vg[2]), fmax3(vg[3], vg[4], vg[5]), fmaxf(vg[6], vg[7]));
-                        // L = |a|^2 - e - 2 M is monotone in M: the group's
-                        // largest M gives its smallest L
-                        Lm[g] = fmaf(-2.f, m, rb);
+                        Mm[g] = fmax3(fmax3(vg[0], vg[1], vg[2]), fmax3(vg[3], vg[4], vg[5]), fmaxf(vg[6], vg[7]));
                     }
-                    const float lmin =
-                        fmin3(fmin3(Lm[0], Lm[1], Lm[2]), fmin3(Lm[3], Lm[4], Lm[5]), fminf(Lm[6], Lm[7]));
-                    if (row_valid && lmin <= fminf(U2, Ush)) {
+                    // L = |a|^2 - e - 2 M is monotone in M: the largest M gives the smallest L
+                    const float mmax = fmax3(fmaxf(Mm[0], Mm[1]), Mm[2], Mm[3]);
+                    if (row_valid && fmaf(-2.f, mmax, rb) <= U2) {
 #pragma unroll
-                        for (int g = 0; g < 8; ++g) {
+                        for (int g = 0; g < 4; ++g) {
                             const float* vg = v + 8 * g;
-                            const float Lmin = Lm[g];
-                            if (Lmin <= fminf(U2, Ush)) {
+                            const float Lmin = fmaf(-2.f, Mm[g], rb);
+                            if (Lmin <= U2) {
                                 // the group's two best columns (largest M
                                 // first): upper bounds for them
                                 float h0 = fmaxf(vg[0], vg[1]), l0 = fminf(vg[0], vg[1]);
@@ -1692,10 +1693,9 @@ __global__ void __launch_bounds__(kThreads, 1) tc_collect(const float* __restric
                                 } else if (Ua < U2) {
                                     U2 = Ua;
                                 }
-                                const float thr = fminf(U2, Ush);
                                 unsigned msk = 0;
 #pragma unroll
-                                for (int j = 0; j < 8; ++j) msk |= (fmaf(-2.f, vg[j], rb) <= thr ? 1u : 0u) << j;
+                                for (int j = 0; j < 8; ++j) msk |= (fmaf(-2.f, vg[j], rb) <= U2 ? 1u : 0u) << j;
                                 while (msk) {
                                     const int j = __ffs(msk) - 1;
                                     msk &= msk - 1;
@@ -1709,34 +1709,27 @@ __global__ void __launch_bounds__(kThreads, 1) tc_collect(const float* __restric
                         }
                     }
                 }
-                *reinterpret_cast<volatile unsigned long long*>(&S.ul[r][wg]) =
-                    (unsigned long long)__float_as_uint(U1) | ((unsigned long long)__float_as_uint(U2) << 32);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&S.empty_a[sa]);  // the row constants are read
             }
             if (!dead && nbuf > 0) flush_cands(row, nbuf);
             nbuf = 0;
-            if (!dead && row_valid) {
-                // lower the row's bound for the items that start later (bounds
-                // are >= 0, so their bits order like integers)
-                const unsigned long long ou = *reinterpret_cast<volatile unsigned long long*>(&S.ul[r][wg ^ 1]);
-                const float ox = __uint_as_float((uint32_t)ou), oy = __uint_as_float((uint32_t)(ou >> 32));
-                const float Uf = fminf(U2, fminf(fmaxf(U1, ox), U1 <= ox ? U2 : oy));
-                if (Uf >= 0.f) atomicMin(reinterpret_cast<int*>(ub + row), __float_as_int(Uf));
-            }
+            // lower the row's bound for the items that start later (bounds
+            // are >= 0, so their bits order like integers)
+            if (!dead && row_valid && U2 >= 0.f) atomicMin(reinterpret_cast<int*>(ub + row), __float_as_int(U2));
         }
     }
     __syncthreads();
     if (*failed) {
         // drain: every issued copy and MMA must land before the memory goes
         // away (each waits for the last phase its barrier has outstanding)
-        if (tid == 32) {
+        if (tid == 9 * 32) {
             for (int st = 0; st < kStages; ++st) {
                 const int last = issued_b - 1 - ((issued_b - 1 - st) % kStages + kStages) % kStages;
                 if (last >= 0 && last % kStages == st) mbar_wait(&S.full_b[st], (last / kStages) & 1);
             }
         }
-        if (tid == 0) {
+        if (tid == 8 * 32) {
             kmx_raise(err, KMX_DERR_TIMEOUT);
             for (int k = 0; k < kAccBufs; ++k) {
                 const int last = issued_mma - 1 - ((issued_mma - 1 - k) % kAccBufs + kAccBufs) % kAccBufs;
@@ -1747,7 +1740,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_collect(const float* __restric
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 0) tmem_dealloc(tmem, kTmemCols);
+    if (warp == 8) tmem_dealloc(tmem, kTmemCols);
 }
 
 // ---------------------------------------------------------------------------
@@ -1875,10 +1868,7 @@ __global__ void __launch_bounds__(256) fallback_merge(const kmx::RowBest* __rest
 
 size_t tc_smem_bytes()
 {
-    // at least 120 KB: one CTA per SM, whose TMEM allocation is all 512
-    // columns (a second CTA would wait in tcgen05.alloc)
-    const size_t need = sizeof(TcShared) + 1024;
-    return need < 120 * 1024 ? 120 * 1024 : need;
+    return sizeof(TcShared) + 1024;
 }
 
 struct TcBuffers {
@@ -2059,14 +2049,14 @@ cudaError_t kmx_match_tc_launch(kmx_ctx* ctx, const float* dp, int64_t np_cap, c
     KMX_COUNT_LAUNCH();
     // about five CTAs per SM fit (registers); more would only wait for the counter
     tc_plan<<<kmx_stride_blocks(tp + tq, 1, ctx->sm_count, 5), kTM, 0, st>>>(planP, planQ, b.nitems + 2);
-    // tensor-core candidates both ways: one persistent CTA per SM
-    const unsigned grid = (unsigned)(ctx->sm_count > 0 ? ctx->sm_count : 1);
+    // tensor-core candidates both ways: persistent CTAs
+    const unsigned grid = (unsigned)(ctx->sm_count > 0 ? kCtasPerSm * ctx->sm_count : 1);
     KMX_COUNT_LAUNCH();
-    tc_collect<<<grid, kThreads, smem, st>>>(dp, permP, np_cap, d_np, b.packQ, b.needP, tq, b.nneedP, b.itemsP,
-                                             b.nitems + 0, b.ubP, b.candP, b.cntP, ctx->d_err);
+    tc_collect<<<grid, kThreads, smem, st>>>(dp, permP, np_cap, d_np, b.packQ, b.needP, tq, b.itemsP, b.nitems + 0,
+                                             b.ubP, b.candP, b.cntP, ctx->d_err);
     KMX_COUNT_LAUNCH();
-    tc_collect<<<grid, kThreads, smem, st>>>(dq, permQ, nq_cap, d_nq, b.packP, b.needQ, tp, b.nneedQ, b.itemsQ,
-                                             b.nitems + 1, b.ubQ, b.candQ, b.cntQ, ctx->d_err);
+    tc_collect<<<grid, kThreads, smem, st>>>(dq, permQ, nq_cap, d_nq, b.packP, b.needQ, tp, b.itemsQ, b.nitems + 1,
+                                             b.ubQ, b.candQ, b.cntQ, ctx->d_err);
     // exact re-ranking; overflowed rows are flagged
     KMX_COUNT_LAUNCH();
     tc_rerank<<<kmx_stride_blocks(np_cap, 32, ctx->sm_count), 256, 0, st>>>(
