@@ -4,13 +4,15 @@
 //
 //   ratio_keys        ratio = d1 / d2 in FP64 (1 when d2 = 0), a 4096-bucket
 //                     histogram of it.
-//   ratio_threshold   one block: the first bucket B at which the cumulative
-//                     count reaches N_tau.
-//   ratio_candidates  the correspondences in buckets <= B (every one of the
-//                     N_tau lowest is among them; all others rank higher).
-//   ratio_rank        each candidate's exact rank among the candidates by
-//                     (ratio, i); ranks < N_tau give the selection in
-//                     ascending order, with both end points gathered.
+//   ratio_threshold   one block: the buckets' first places and the first
+//                     bucket B at which the cumulative count reaches N_tau.
+//   ratio_candidates  the correspondences in buckets <= B, bucket by bucket
+//                     (every one of the N_tau lowest is among them; all others
+//                     rank higher).
+//   ratio_rank        each candidate's exact rank by (ratio, i) among its
+//                     bucket's, after the buckets below; ranks < N_tau give
+//                     the selection in ascending order, with both end points
+//                     gathered.
 //   graph_build       one 32-bit word of the adjacency bit matrix per thread:
 //                     k ~ k' iff | |b_k - b_k'| - |a_k - a_k'| | <= 2 beta.  The
 //                     test runs in FP32; within a band around the threshold it
@@ -21,11 +23,11 @@
 //                     point of c(v) <- H({c(u) : u ~ v}) started from the
 //                     degrees (H = h-index: the largest h with at least h
 //                     values >= h; the values only decrease and stay above the
-//                     core numbers, so in-place updates converge to them),
-//                     sweeps separated by a bounded grid barrier, until a
-//                     sweep changes nothing; then the largest core number
-//                     and the positions of the maximum k-core in ascending
-//                     order.
+//                     core numbers, so updates in any order converge to them).
+//                     Rounds of kPasses passes over the vertices, separated by
+//                     a bounded grid barrier, until a round changes nothing;
+//                     then the largest core number and the positions of the
+//                     maximum k-core in ascending order.
 #include "kmx_internal.cuh"
 
 #include <cooperative_groups.h>
@@ -35,23 +37,27 @@ namespace {
 constexpr int kBuckets = 4096;
 constexpr int kThreads = 256;
 constexpr uint32_t kSpinLimit = 1u << 24;
-constexpr int kMaxSweeps = 1 << 16;
-constexpr int kHistCap = 2048;  // per-warp histogram of capped neighbour values (values below it)
+constexpr int kMaxRounds = 1 << 16;
+constexpr int kCoreThreads = 1024;
+constexpr int kCoreWarps = kCoreThreads / 32;
+constexpr int kPasses = 4;                  // passes between two grid barriers
+constexpr size_t kCoreSmem = 136 * 1024;    // snapshot, vertex states and neighbour lists of a kcore CTA
 
 struct PruneScratch {
     double* ratio;            // [n_cap]
     int32_t* bucket;          // [n_cap]
-    int32_t* hist;            // [kBuckets]
+    int32_t* hist;            // [kBuckets] counts, then the places left to fill
+    int32_t* first;           // [kBuckets + 1] first place of each bucket; from the last candidate bucket on, their number
     int32_t* cand;            // [n_cap]
     unsigned long long* ckey; // [n_cap] candidate ratio bits
     int32_t* ci;              // [n_cap] candidate source index i
-    int32_t* n_cand;          // [1]
     int32_t* thr;             // [1] threshold bucket
+    int32_t* odd;             // [1] some ratio's bits do not order like its bucket (NaN or a set sign)
     float4* pa;               // [n_tau] source end point of each selected correspondence
     float4* pb;               // [n_tau] target end point
     uint32_t* adj;            // [n_tau][words]
-    int32_t* core;            // [n_tau] working values (copied to the caller)
-    uint32_t* sync;           // [8] barrier count, barrier generation, change counters x3, work counters x3
+    uint16_t* core;           // [n_tau, padded to 8] working values
+    uint32_t* sync;           // [2] barrier arrivals (changed blocks in the high half), barrier generation
 };
 
 __device__ __forceinline__ int64_t corr_count(const int64_t* d_n, int64_t cap)
@@ -72,37 +78,46 @@ __global__ void __launch_bounds__(kThreads) ratio_keys(const kmx_corr* __restric
         int b = (int)(r * (double)kBuckets);  // r in [0, 1]; exact scaling by a power of two
         b = b < 0 ? 0 : (b >= kBuckets ? kBuckets - 1 : b);
         s.bucket[k] = b;
+        if (!(r >= 0.0) || signbit(r)) *s.odd = 1;
         atomicAdd(&s.hist[b], 1);
     }
 }
 
-__global__ void __launch_bounds__(1024) ratio_threshold(int32_t n_tau, PruneScratch s)
+// exclusive prefix over the CTA's 1024 threads
+__device__ __forceinline__ int32_t block_prefix(int32_t x, int32_t* wsum)
 {
-    __shared__ int32_t part[1024];
-    constexpr int kPer = kBuckets / 1024;
-    int32_t loc = 0;
-    for (int e = 0; e < kPer; ++e) loc += s.hist[threadIdx.x * kPer + e];
-    part[threadIdx.x] = loc;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int32_t inc = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) wsum[warp] = inc;
     __syncthreads();
-    // inclusive prefix over the 1024 partial sums (Hillis-Steele)
-    for (int o = 1; o < 1024; o <<= 1) {
-        const int32_t v = threadIdx.x >= (unsigned)o ? part[threadIdx.x - o] : 0;
-        __syncthreads();
-        part[threadIdx.x] += v;
-        __syncthreads();
+    int32_t before = 0;
+    if (lane < warp) before = wsum[lane];
+    before = __reduce_add_sync(0xffffffffu, before);
+    return before + inc - x;
+}
+
+__global__ void __launch_bounds__(1024) ratio_threshold(const int64_t* d_n, int64_t cap, int32_t n_tau, PruneScratch s,
+                                                        int64_t* __restrict__ n_sel)
+{
+    __shared__ int32_t wsum[32];
+    constexpr int kPer = kBuckets / 1024;
+    static_assert(kPer == 4, "one int4 per thread");
+    const int4 h = reinterpret_cast<const int4*>(s.hist)[threadIdx.x];
+    const int32_t f0 = block_prefix(h.x + h.y + h.z + h.w, wsum);
+    const int32_t f1 = f0 + h.x, f2 = f1 + h.y, f3 = f2 + h.z, f4 = f3 + h.w;
+    reinterpret_cast<int4*>(s.first)[threadIdx.x] = make_int4(f0, f1, f2, f3);
+    if (threadIdx.x == 1023) {
+        s.first[kBuckets] = f4;
+        if (f4 < n_tau) *s.thr = kBuckets - 1;  // fewer than N_tau in all
+        const int64_t n = corr_count(d_n, cap);
+        *n_sel = n < n_tau ? n : n_tau;
     }
-    const int32_t before = threadIdx.x ? part[threadIdx.x - 1] : 0;
-    if (threadIdx.x == 1023 && part[1023] < n_tau) *s.thr = kBuckets - 1;  // fewer than N_tau in all
-    if (before < n_tau && part[threadIdx.x] >= n_tau) {
-        int32_t c = before;
-        for (int e = 0; e < kPer; ++e) {
-            c += s.hist[threadIdx.x * kPer + e];
-            if (c >= n_tau) {
-                *s.thr = threadIdx.x * kPer + e;
-                break;
-            }
-        }
-    }
+    if (f0 < n_tau && f4 >= n_tau) *s.thr = threadIdx.x * kPer + (f1 >= n_tau ? 0 : f2 >= n_tau ? 1 : f3 >= n_tau ? 2 : 3);
 }
 
 __global__ void __launch_bounds__(kThreads) ratio_candidates(const kmx_corr* __restrict__ corr, int64_t cap,
@@ -110,13 +125,14 @@ __global__ void __launch_bounds__(kThreads) ratio_candidates(const kmx_corr* __r
 {
     const int64_t n = corr_count(d_n, cap);
     const int32_t thr = *s.thr;
-    for (int64_t k = (int64_t)blockIdx.x * kThreads + threadIdx.x; k < n; k += (int64_t)gridDim.x * kThreads)
-        if (s.bucket[k] <= thr) {
-            const int c = atomicAdd(s.n_cand, 1);
-            s.cand[c] = (int32_t)k;
-            s.ckey[c] = (unsigned long long)__double_as_longlong(s.ratio[k]);
-            s.ci[c] = corr[k].i;
-        }
+    for (int64_t k = (int64_t)blockIdx.x * kThreads + threadIdx.x; k < n; k += (int64_t)gridDim.x * kThreads) {
+        const int b = s.bucket[k];
+        if (b > thr) continue;
+        const int c = s.first[b] + atomicSub(&s.hist[b], 1) - 1;
+        s.cand[c] = (int32_t)k;
+        s.ckey[c] = (unsigned long long)__double_as_longlong(s.ratio[k]);
+        s.ci[c] = corr[k].i;
+    }
 }
 
 // (ratio, i) lexicographic: a non-negative double orders like its bits.
@@ -125,31 +141,43 @@ __device__ __forceinline__ bool key_less(unsigned long long ra, int32_t ia, unsi
     return ra < rb || (ra == rb && ia < ib);
 }
 
-// One warp per candidate: its rank among the candidates (the lanes stride
-// over the compact keys).
+// One warp per candidate: its rank among its bucket's (the lanes stride over
+// the compact keys), after the buckets below.
 __global__ void __launch_bounds__(kThreads) ratio_rank(const kmx_corr* __restrict__ corr, int32_t n_tau,
                                                       const float4* __restrict__ src4,
                                                       const float4* __restrict__ tgt4, PruneScratch s,
                                                       int32_t* __restrict__ sel)
 {
-    const int m = *s.n_cand;
+    const int m = s.first[*s.thr + 1];
     const int lane = threadIdx.x & 31;
     const int warps = gridDim.x * (kThreads / 32);
     for (int c = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); c < m; c += warps) {
+        const int32_t k = s.cand[c];
         const unsigned long long rk = s.ckey[c];
         const int32_t ik = s.ci[c];
+        const kmx_corr e = corr[k];
+        const int b = s.bucket[k];
+        const bool odd = *s.odd != 0;
+        const int f0 = odd ? 0 : s.first[b], f1 = odd ? m : s.first[b + 1];
         int rank = 0;
-        for (int f = lane; f < m; f += 32) rank += key_less(s.ckey[f], s.ci[f], rk, ik);
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
-        if (lane == 0 && rank < n_tau) {
-            const int32_t k = s.cand[c];
-            sel[rank] = k;
-            const kmx_corr e = corr[k];
-            s.pa[rank] = src4[e.i];
-            s.pb[rank] = tgt4[e.j];
+        for (int f = f0 + lane; f < f1; f += 32) rank += key_less(s.ckey[f], s.ci[f], rk, ik);
+        rank = f0 + __reduce_add_sync(0xffffffffu, rank);
+        if (rank < n_tau) {
+            if (lane == 0) {
+                sel[rank] = k;
+                s.pa[rank] = src4[e.i];
+            } else if (lane == 1) {
+                s.pb[rank] = tgt4[e.j];
+            }
         }
     }
+}
+
+__device__ __forceinline__ float sqrt_approx(float x)
+{
+    float y;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
 
 __device__ __forceinline__ bool edge_fp64(float4 a, float4 a2, float4 b, float4 b2, double two_beta)
@@ -161,8 +189,7 @@ __device__ __forceinline__ bool edge_fp64(float4 a, float4 a2, float4 b, float4 
     return fabs(__dadd_rn(db, -da)) <= two_beta;
 }
 
-// Thread (v, w): bits u = 32 w .. 32 w + 31 of row v.  The degree of v is the
-// popcount of its row.
+// Thread (v, w): bits u = 32 w .. 32 w + 31 of row v.
 __global__ void __launch_bounds__(kThreads) graph_build(int32_t n_tau, const int64_t* d_n_sel, double two_beta,
                                                        PruneScratch s, int32_t words)
 {
@@ -180,10 +207,12 @@ __global__ void __launch_bounds__(kThreads) graph_build(int32_t n_tau, const int
             const float4 a2 = s.pa[u], b2 = s.pb[u];
             const float ax = a.x - a2.x, ay = a.y - a2.y, az = a.z - a2.z;
             const float bx = b.x - b2.x, by = b.y - b2.y, bz = b.z - b2.z;
-            const float da = sqrtf(fmaf(az, az, fmaf(ay, ay, ax * ax)));
-            const float db = sqrtf(fmaf(bz, bz, fmaf(by, by, bx * bx)));
+            const float da = sqrt_approx(fmaf(az, az, fmaf(ay, ay, ax * ax)));
+            const float db = sqrt_approx(fmaf(bz, bz, fmaf(by, by, bx * bx)));
             const float gap = fabsf(db - da) - tb;
-            // FP32 carries a few ulp of the distances; decide again in FP64 near the threshold
+            // FP32 carries a few ulp of the distances (the approximate root,
+            // which halves the instructions of a pair, one more); decide again
+            // in FP64 near the threshold
             const float band = 1e-5f * (1.0f + da + db);
             bool on;
             if (gap > band)
@@ -195,211 +224,214 @@ __global__ void __launch_bounds__(kThreads) graph_build(int32_t n_tau, const int
             bits |= (uint32_t)on << e;
         }
         s.adj[(int64_t)v * words + w] = bits;
-        if (bits) atomicAdd(&s.core[v], __popc(bits));
     }
 }
 
 __device__ __forceinline__ uint32_t ld_volatile(const uint32_t* p) { return *reinterpret_cast<const volatile uint32_t*>(p); }
 
-// Bounded grid barrier (sense by generation); false when a spin ran out.
-__device__ bool grid_barrier(uint32_t* count, uint32_t* gen, uint32_t nblocks)
+// Bounded grid barrier (generation `round` + 1 once every block has arrived);
+// `changed` of any block reaches all of them as *any.  False when a spin ran out.
+__device__ bool grid_barrier(uint32_t* sync, uint32_t nblocks, uint32_t round, bool changed, bool* any)
 {
-    __shared__ int ok;
-    __syncthreads();
+    __shared__ uint32_t state;
+    const int mine = __syncthreads_or(changed);
     if (threadIdx.x == 0) {
-        ok = 1;
-        const uint32_t g = ld_volatile(gen);
+        const uint32_t want = round + 1;
+        uint32_t seen;
         __threadfence();
-        if (atomicAdd(count, 1u) == nblocks - 1) {
-            atomicExch(count, 0u);
+        const uint32_t add = mine ? 0x10001u : 1u;
+        const uint32_t sum = atomicAdd(sync, add) + add;
+        if ((sum & 0xffffu) == nblocks) {
+            seen = want | (sum >> 16 ? 0x80000000u : 0u);
+            atomicExch(sync, 0u);
             __threadfence();
-            atomicAdd(gen, 1u);
+            atomicExch(sync + 1, seen);
         } else {
             uint32_t it = 0;
-            while (ld_volatile(gen) == g) {
+            while (((seen = ld_volatile(sync + 1)) & 0x7fffffffu) != want) {
                 if (++it > kSpinLimit) {
-                    ok = 0;
+                    seen = 0xffffffffu;
                     break;
                 }
             }
         }
         __threadfence();
+        state = seen;
     }
     __syncthreads();
-    return ok != 0;
+    const uint32_t st = state;
+    *any = (st >> 31) != 0;
+    return st != 0xffffffffu;
 }
 
-// count of neighbours u of v with c(u) >= h over the block's snapshot of c
-// (warp-wide, every lane gets it)
-__device__ __forceinline__ int count_ge(const uint32_t* __restrict__ row, int words, const int32_t* snap, int h)
-{
-    int cnt = 0;
-    for (int w = threadIdx.x & 31; w < words; w += 32) {
-        uint32_t bits = row[w];
-        while (bits) {
-            const int e = __ffs(bits) - 1;
-            bits &= bits - 1;
-            cnt += snap[w * 32 + e] >= h;
-        }
-    }
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-    return cnt;
-}
+// values of a snapshot: n_tau rounded up to whole words of the bit rows
+__host__ __device__ constexpr int32_t snap_len(int32_t n_tau) { return (n_tau + 31) / 32 * 32; }
 
-__global__ void __launch_bounds__(kThreads) kcore(const int64_t* d_n_sel, int32_t words, PruneScratch s,
-                                                 int32_t* __restrict__ core_out, int32_t* __restrict__ kmax_out,
-                                                 int32_t* __restrict__ inlier, int64_t* __restrict__ n_inlier,
-                                                 unsigned int* __restrict__ err)
+struct CoreVertex {
+    int32_t c;      // current value
+    int32_t deg;
+    int32_t start;  // of the neighbour list in the warp's part, -1: the list did not fit
+};
+
+// number of neighbours u of the vertex with snap[u] >= h (warp-wide, every lane
+// gets it): over its list, or over its bit row
+__device__ __forceinline__ int count_ge(const uint16_t* list, int deg, const uint32_t* __restrict__ row, int words,
+                                        const uint16_t* snap, int h)
 {
-    const int nsel = (int)*d_n_sel;
-    const uint32_t nblocks = gridDim.x;
     const int lane = threadIdx.x & 31;
-    int32_t* c = s.core;
-    uint32_t* bar_count = s.sync;
-    uint32_t* bar_gen = s.sync + 1;
-    uint32_t* changed = s.sync + 2;  // three rotating counters
-    // dynamic shared memory: per-warp histograms of kHistCap ints, then the
-    // snapshot of c taken at the start of each sweep
-    extern __shared__ int32_t dyn[];
-    int32_t* hist = dyn + (threadIdx.x >> 5) * kHistCap;
-    int32_t* snap = dyn + (kThreads / 32) * kHistCap;
-    uint32_t* work = s.sync + 5;  // three rotating per-sweep vertex counters
-    __shared__ uint32_t block_changed;
-    bool ok = true;
-    for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
-        if (threadIdx.x == 0) block_changed = 0;
-        for (int v = threadIdx.x; v < nsel; v += kThreads) snap[v] = *reinterpret_cast<const volatile int32_t*>(&c[v]);
-        __syncthreads();
-        while (true) {
-            int v = 0;
-            if (lane == 0) v = (int)atomicAdd(&work[sweep % 3], 1u);
-            v = __shfl_sync(0xffffffffu, v, 0);
-            if (v >= nsel) break;
-            const int cv = snap[v];
-            if (cv == 0) continue;
-            const uint32_t* row = s.adj + (int64_t)v * words;
-            int h = cv;
-            if (count_ge(row, words, snap, cv) < cv) {
-                if (cv < kHistCap) {
-                    // histogram of min(c(u), cv), then the largest h with at
-                    // least h values >= h, scanning 32 h's at a time from cv down
-                    for (int e = lane; e <= cv; e += 32) hist[e] = 0;
-                    __syncwarp();
-                    for (int w = lane; w < words; w += 32) {
-                        uint32_t bits = row[w];
-                        while (bits) {
-                            const int b = __ffs(bits) - 1;
-                            bits &= bits - 1;
-                            atomicAdd(&hist[min(snap[w * 32 + b], cv)], 1);
-                        }
-                    }
-                    __syncwarp();
-                    int suffix = 0;
-                    for (int top = cv;; top -= 32) {
-                        const int hh = top - lane;
-                        int x = hh >= 0 ? hist[hh] : 0;
-#pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) {
-                            const int y = __shfl_up_sync(0xffffffffu, x, o);
-                            if (lane >= o) x += y;
-                        }
-                        const unsigned hit = __ballot_sync(0xffffffffu, hh >= 0 && suffix + x >= hh);
-                        if (hit) {
-                            h = top - (__ffs(hit) - 1);
-                            break;
-                        }
-                        suffix += __shfl_sync(0xffffffffu, x, 31);
-                    }
-                    __syncwarp();
-                } else {
-                    // the largest h < cv with count_ge(h) >= h (count_ge falls as h grows)
-                    int lo = 0, hi = cv - 1;
-                    while (lo < hi) {
-                        const int mid = (lo + hi + 1) >> 1;
-                        if (count_ge(row, words, snap, mid) >= mid)
-                            lo = mid;
-                        else
-                            hi = mid - 1;
-                    }
-                    h = lo;
-                }
-            }
-            if (h != cv) {
-                if (lane == 0) {
-                    *reinterpret_cast<volatile int32_t*>(&c[v]) = h;
-                    atomicAdd(&block_changed, 1u);
-                }
+    int cnt = 0;
+    if (list) {
+#pragma unroll 4
+        for (int e = lane; e < deg; e += 32) cnt += snap[list[e]] >= h;
+    } else {
+        for (int w = lane; w < words; w += 32) {
+            uint32_t bits = row[w];
+            while (bits) {
+                const int e = __ffs(bits) - 1;
+                bits &= bits - 1;
+                cnt += snap[w * 32 + e] >= h;
             }
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            if (block_changed) atomicAdd(&changed[sweep % 3], block_changed);
-            if (blockIdx.x == 0) {
-                changed[(sweep + 1) % 3] = 0;
-                work[(sweep + 1) % 3] = 0;
-            }
-        }
-        if (!grid_barrier(bar_count, bar_gen, nblocks)) {
-            ok = false;
-            break;
-        }
-        if (ld_volatile(&changed[sweep % 3]) == 0) break;
     }
-    if (!ok) {
-        if (threadIdx.x == 0) kmx_raise(err, KMX_DERR_TIMEOUT);
+    return __reduce_add_sync(0xffffffffu, cnt);
+}
+
+// One warp per vertex (per_warp of them at most), whose neighbour list it keeps
+// in shared memory as 16-bit indices.  A pass reads all values (2 n bytes from
+// L2) and lowers the CTA's own; passes of different CTAs are not ordered, and
+// only the barrier after kPasses of them decides whether anything still moves
+// (a round without a change saw the same values in all its passes).  What
+// bounds it: the L2 round trip of a pass and the barrier's.  Before, a pass took
+// vertices from a global counter, walked 32-bit rows in L2 and ended in a
+// barrier: 3000 vertices of 160 neighbours took 1042 us, now 263 us.
+__global__ void __launch_bounds__(kCoreThreads, 1) kcore(const int64_t* d_n_sel, int32_t words, int32_t per_warp,
+                                                         int32_t list_len, PruneScratch s,
+                                                         int32_t* __restrict__ core_out, int32_t* __restrict__ kmax_out,
+                                                         int32_t* __restrict__ inlier, int64_t* __restrict__ n_inlier,
+                                                         unsigned int* __restrict__ err)
+{
+    const int n = (int)*d_n_sel;
+    const uint32_t nblocks = gridDim.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // dynamic shared memory: the values at the start of a pass, the warps'
+    // vertices, their neighbour lists
+    extern __shared__ __align__(16) uint8_t dyn[];
+    uint16_t* snap = reinterpret_cast<uint16_t*>(dyn);
+    const int n8 = (n + 7) / 8;
+    CoreVertex* vert = reinterpret_cast<CoreVertex*>(dyn + sizeof(uint16_t) * snap_len(words * 32));
+    uint16_t* list = reinterpret_cast<uint16_t*>(vert + kCoreWarps * per_warp) + (size_t)warp * list_len;
+    vert += warp * per_warp;
+    // vertex k of the warp
+    const int step = kCoreWarps * (int)nblocks, v0 = warp * (int)nblocks + (int)blockIdx.x;
+    int used = 0;
+    for (int k = 0, v = v0; v < n; ++k, v += step) {
+        const uint32_t* row = s.adj + (int64_t)v * words;
+        int deg = 0;
+        for (int w0 = 0; w0 < words; w0 += 32) {
+            uint32_t bits = w0 + lane < words ? row[w0 + lane] : 0u;
+            const int mine = __popc(bits);
+            int inc = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += y;
+            }
+            int at = used + deg + inc - mine;
+            while (bits) {
+                const int e = __ffs(bits) - 1;
+                bits &= bits - 1;
+                if (at < list_len) list[at] = (uint16_t)((w0 + lane) * 32 + e);
+                ++at;
+            }
+            deg += __shfl_sync(0xffffffffu, inc, 31);
+        }
+        const bool fits = used + deg <= list_len;
+        if (lane == 0) {
+            vert[k] = CoreVertex{deg, deg, fits ? used : -1};
+            *reinterpret_cast<volatile uint16_t*>(s.core + v) = (uint16_t)deg;
+        }
+        if (fits) used += deg;
+        __syncwarp();
+    }
+    bool any = false;
+    bool ok = grid_barrier(s.sync, nblocks, 0, false, &any);
+    for (uint32_t round = 1; ok && round <= kMaxRounds; ++round) {
+        bool changed = false;
+        for (int pass = 0; pass < kPasses; ++pass) {
+            for (int i = tid; i < n8; i += kCoreThreads) {
+                uint4 q;
+                asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];"
+                             : "=r"(q.x), "=r"(q.y), "=r"(q.z), "=r"(q.w)
+                             : "l"(reinterpret_cast<const uint4*>(s.core) + i)
+                             : "memory");
+                reinterpret_cast<uint4*>(snap)[i] = q;
+            }
+            __syncthreads();
+            for (int k = 0, v = v0; v < n; ++k, v += step) {
+                const CoreVertex x = vert[k];
+                if (x.c == 0) continue;
+                const uint32_t* row = s.adj + (int64_t)v * words;
+                const uint16_t* nb = x.start >= 0 ? list + x.start : nullptr;
+                // count_ge falls as h grows: with `lo` values >= c, at least
+                // `lo` are >= lo
+                int lo = count_ge(nb, x.deg, row, words, snap, x.c);
+                if (lo >= x.c) continue;
+                int hi = x.c - 1;
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (count_ge(nb, x.deg, row, words, snap, mid) >= mid)
+                        lo = mid;
+                    else
+                        hi = mid - 1;
+                }
+                if (lane == 0) {
+                    vert[k].c = lo;
+                    *reinterpret_cast<volatile uint16_t*>(s.core + v) = (uint16_t)lo;
+                }
+                __syncwarp();
+                changed = true;
+            }
+            __syncthreads();  // the values are read before the next pass overwrites them
+        }
+        ok = grid_barrier(s.sync, nblocks, round, changed, &any);
+        if (!any) break;
+    }
+    if (!ok || any) {
+        if (tid == 0) kmx_raise(err, KMX_DERR_TIMEOUT);
         return;
     }
     if (blockIdx.x != 0) return;
     // block 0: largest core number, then the maximum k-core in ascending order
-    __shared__ int32_t red[kThreads];
-    __shared__ int32_t base;
+    // (the last round changed nothing: snap holds the core numbers)
+    __shared__ int32_t wsum[kCoreWarps];
     int32_t mx = 0;
-    for (int v = threadIdx.x; v < nsel; v += kThreads) {
-        const int32_t cv = *reinterpret_cast<const volatile int32_t*>(&c[v]);
+    for (int v = tid; v < n; v += kCoreThreads) {
+        const int32_t cv = snap[v];
         core_out[v] = cv;
         mx = max(mx, cv);
     }
-    red[threadIdx.x] = mx;
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) wsum[warp] = mx;
     __syncthreads();
-    for (int o = kThreads / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < (unsigned)o) red[threadIdx.x] = max(red[threadIdx.x], red[threadIdx.x + o]);
-        __syncthreads();
+    const int32_t kmax = __reduce_max_sync(0xffffffffu, wsum[lane]);
+    __syncthreads();
+    int32_t base = 0;
+    for (int b = 0; b < n; b += kCoreThreads) {
+        const int v = b + tid;
+        const bool in = v < n && snap[v] == kmax;
+        const int32_t at = base + block_prefix(in, wsum);
+        if (in) inlier[at] = v;
+        base += __syncthreads_count(in);
     }
-    const int32_t kmax = red[0];
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         *kmax_out = kmax;
-        base = 0;
+        *n_inlier = base;
     }
-    __syncthreads();
-    for (int v0 = 0; v0 < nsel; v0 += kThreads) {
-        const int v = v0 + threadIdx.x;
-        const bool in = v < nsel && nsel > 0 && *reinterpret_cast<const volatile int32_t*>(&c[v]) == kmax;
-        const unsigned bal = __ballot_sync(0xffffffffu, in);
-        __shared__ int32_t wcount[kThreads / 32];
-        if (lane == 0) wcount[threadIdx.x >> 5] = __popc(bal);
-        __syncthreads();
-        int off = base;
-        for (int w = 0; w < (int)(threadIdx.x >> 5); ++w) off += wcount[w];
-        if (in) inlier[off + __popc(bal & ((1u << lane) - 1u))] = v;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int tot = 0;
-            for (int w = 0; w < kThreads / 32; ++w) tot += wcount[w];
-            base += tot;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *n_inlier = base;
-}
-
-__global__ void set_n_sel(const int64_t* d_n, int64_t cap, int32_t n_tau, int64_t* n_sel)
-{
-    const int64_t n = corr_count(d_n, cap);
-    *n_sel = n < n_tau ? n : n_tau;
 }
 
 int32_t words_for(int32_t n_tau) { return (n_tau + 31) / 32; }
+
+size_t zero_bytes() { return sizeof(int32_t) * (kBuckets + 2 + 2); }
 
 PruneScratch carve(void* base, int64_t cap, int32_t n_tau, size_t* total)
 {
@@ -413,19 +445,17 @@ PruneScratch carve(void* base, int64_t cap, int32_t n_tau, size_t* total)
     s.pa = static_cast<float4*>(a.take(sizeof(float4) * (n_tau + 1)));
     s.pb = static_cast<float4*>(a.take(sizeof(float4) * (n_tau + 1)));
     s.adj = static_cast<uint32_t*>(a.take(sizeof(uint32_t) * ((size_t)n_tau * words_for(n_tau) + 1)));
-    // zeroed together: histogram, candidate count, threshold, core (degree) counters, sync words
-    const size_t zero_words = kBuckets + 2 + (size_t)n_tau + 8;
-    int32_t* z = static_cast<int32_t*>(a.take(sizeof(int32_t) * zero_words));
+    s.first = static_cast<int32_t*>(a.take(sizeof(int32_t) * (kBuckets + 1)));
+    s.core = static_cast<uint16_t*>(a.take(sizeof(uint16_t) * (size_t)snap_len(n_tau)));
+    // zeroed together: histogram, threshold, odd flag, sync words
+    int32_t* z = static_cast<int32_t*>(a.take(zero_bytes()));
     s.hist = z;
-    s.n_cand = z + kBuckets;
-    s.thr = z + kBuckets + 1;
-    s.core = z + kBuckets + 2;
-    s.sync = reinterpret_cast<uint32_t*>(z + kBuckets + 2 + n_tau);
+    s.thr = z + kBuckets;
+    s.odd = z + kBuckets + 1;
+    s.sync = reinterpret_cast<uint32_t*>(z + kBuckets + 2);
     *total = kmx_align_up(a.used, 256);
     return s;
 }
-
-size_t zero_bytes(int32_t n_tau) { return sizeof(int32_t) * (kBuckets + 2 + (size_t)n_tau + 8); }
 
 }  // namespace
 
@@ -445,14 +475,12 @@ cudaError_t kmx_prune_launch(kmx_ctx* ctx, const kmx_corr* corr, int64_t cap, co
     size_t total = 0;
     PruneScratch s = carve(scratch, cap, n_tau, &total);
     cudaError_t e;
-    if ((e = cudaMemsetAsync(s.hist, 0, zero_bytes(n_tau), st))) return e;
+    if ((e = cudaMemsetAsync(s.hist, 0, zero_bytes(), st))) return e;
     const unsigned grid = 4u * (unsigned)ctx->sm_count;
-    KMX_COUNT_LAUNCH();
-    set_n_sel<<<1, 1, 0, st>>>(d_n, cap, n_tau, n_sel);
     KMX_COUNT_LAUNCH();
     ratio_keys<<<grid, kThreads, 0, st>>>(corr, cap, d_n, s);
     KMX_COUNT_LAUNCH();
-    ratio_threshold<<<1, 1024, 0, st>>>(n_tau, s);
+    ratio_threshold<<<1, 1024, 0, st>>>(d_n, cap, n_tau, s, n_sel);
     KMX_COUNT_LAUNCH();
     ratio_candidates<<<grid, kThreads, 0, st>>>(corr, cap, d_n, s);
     KMX_COUNT_LAUNCH();
@@ -460,23 +488,23 @@ cudaError_t kmx_prune_launch(kmx_ctx* ctx, const kmx_corr* corr, int64_t cap, co
     const int32_t words = words_for(n_tau);
     KMX_COUNT_LAUNCH();
     graph_build<<<grid, kThreads, 0, st>>>(n_tau, n_sel, 2.0 * beta, s, words);
-    // one CTA per SM (co-resident under a cooperative launch: the sweeps wait
+    // one CTA per SM (co-resident under a cooperative launch: the rounds wait
     // on one another through the grid barrier)
-    const size_t snap_bytes = sizeof(int32_t) * ((size_t)n_tau + (size_t)(kThreads / 32) * kHistCap);
-    // this call is never captured (cooperative launch), so the opt-in is set
-    // to the exact size on every call
-    if (snap_bytes > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(kcore, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)snap_bytes)))
-        return e;
-    int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kcore, kThreads, snap_bytes))) return e;
-    if (per_sm < 1) return cudaErrorLaunchOutOfResources;
     const unsigned kgrid = (unsigned)ctx->sm_count;
+    const int per_warp = (n_tau + kCoreWarps * (int)kgrid - 1) / (kCoreWarps * (int)kgrid);
+    const size_t fixed = sizeof(uint16_t) * (size_t)snap_len(n_tau) + sizeof(CoreVertex) * kCoreWarps * (size_t)per_warp;
+    // 16384 vertices of four a warp take 34 KB of it
+    const size_t smem = kCoreSmem > fixed ? kCoreSmem : fixed;
+    const int list_len = (int)((smem - fixed) / (sizeof(uint16_t) * kCoreWarps));
+    if ((e = kmx_once_per_device(kmx_attr_kcore, [] {
+            return cudaFuncSetAttribute(kcore, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024);
+        })))
+        return e;
     const int64_t* n_sel_c = n_sel;
-    int32_t words_c = words;
+    int32_t words_c = words, per_warp_c = per_warp, list_len_c = list_len;
     unsigned int* err = ctx->d_err;
-    void* args[] = {(void*)&n_sel_c, (void*)&words_c, (void*)&s, (void*)&core_out, (void*)&kmax, (void*)&inlier,
-                    (void*)&n_inlier, (void*)&err};
+    void* args[] = {(void*)&n_sel_c, (void*)&words_c, (void*)&per_warp_c, (void*)&list_len_c, (void*)&s, (void*)&core_out,
+                    (void*)&kmax, (void*)&inlier, (void*)&n_inlier, (void*)&err};
     KMX_COUNT_LAUNCH();
-    return cudaLaunchCooperativeKernel((const void*)kcore, dim3(kgrid), dim3(kThreads), args, snap_bytes, st);
+    return cudaLaunchCooperativeKernel((const void*)kcore, dim3(kgrid), dim3(kCoreThreads), args, smem, st);
 }
