@@ -6,14 +6,22 @@
 // One CTA per problem (the maximum k-core holds a few thousand
 // correspondences).  The points sit in shared memory, centred on their
 // unweighted centroids (taken in FP64), so the FP32 residuals and moments
-// carry only the spread of the cloud; the block reductions end in FP64 in one
-// warp; the 4 x 4 symmetric eigenproblem of Horn's method is solved by cyclic
-// Jacobi in thread 0.  The GNC schedule is the one of the paper's solver:
+// carry only the spread of the cloud; the block reductions end in FP64.  The
+// GNC schedule is the one of the paper's solver:
 // weights w = 1 first; mu = c^2 / (2 r_max^2 - c^2); each iteration sets
 // w = 1 for r^2 <= mu/(mu+1) c^2, 0 for r^2 >= (mu+1)/mu c^2 and
 // c sqrt(mu (mu+1)) / r - mu between, refits, and multiplies mu by the
 // factor; it stops when fewer than 3 weights are positive (keeping the
 // previous fit) or when the weighted cost repeats within tol.
+//
+// What bounds it: one CTA's serial chain.  An FP64 instruction occupies its
+// pipe for tens of cycles whatever the number of active lanes, so FP64 work is
+// laid across lanes and out of the threads that do not need it: the schedule's
+// roots and divisions for 32 iterations at a time (they do not depend on the
+// data), the warp sums' tree with a few lanes per total, centroids, covariance
+// and rotation with a lane per entry.  One pass over the points per iteration
+// forms the residuals, the cost of the last fit, the next weights and their
+// moments, with one reduction.  269 points, 22 iterations: 570 -> 203 us.
 #include "kmx_internal.cuh"
 
 namespace {
@@ -29,37 +37,73 @@ struct GncOut {
     int32_t* stats;  // [4]: iterations, weights > 0.5, points, status (0 ok, 1 fewer than 3 points, 2 too many)
 };
 
-// Sum of up to 16 per-thread FP32 values over the block (warp sums in FP32,
-// the kWarpsG warp sums added in FP64 by warp 0); every thread gets the
-// totals in tot[].
-template <int N>
-__device__ __forceinline__ void block_sum(const float (&v)[N], double* red, double (&tot)[N])
+constexpr int kSums = 18;  // 16 moments, the weighted cost, the positive weights
+
+struct Shared {
+    float part[kWarpsG][kSums + 1];  // warp sums (stride 19: no bank conflicts)
+    double tot[kSums];               // block sums
+    float4 sched[32];                // lo, hi, c sqrt(mu (mu+1)), mu of 32 iterations
+    float R[9];                      // current rotation (FP32, for the residuals)
+    float tc[3];                     // translation in the centred frame: b' = R a' + tc
+    double Rd[9];                    // current rotation, FP64 copy for the output
+    double ca[6];                    // weighted centroids of a and b
+    float H[9];                      // weighted cross-covariance
+    float q[4];                      // the quaternion
+    int32_t count[kWarpsG];
+};
+
+// One step of a warp's sum of N values per lane: the lanes with bit O keep the
+// upper half of the values, the others the lower half, each added to the other
+// side's.  After O = 16, 8, 4, 2, 1 from 16 values lane pairs hold one whole sum
+// each, added in the order of a butterfly over every value.
+template <int N, int O>
+__device__ __forceinline__ void sum_step(float (&v)[16], int lane)
+{
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+        const bool up = (lane & O) != 0;
+        const float keep = up ? v[i + N / 2] : v[i], give = up ? v[i] : v[i + N / 2];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, give, O);
+    }
+}
+
+// Warp sums of v[0..15], cost and npos into S.part[warp].
+__device__ __forceinline__ void warp_sums(float (&v)[16], float cost, float npos, Shared& S)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float x[N];
+    sum_step<16, 16>(v, lane);
+    sum_step<8, 8>(v, lane);
+    sum_step<4, 4>(v, lane);
+    sum_step<2, 2>(v, lane);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
 #pragma unroll
-    for (int i = 0; i < N; ++i) {
-        x[i] = v[i];
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) x[i] += __shfl_xor_sync(0xffffffffu, x[i], o);
+    for (int o = 16; o >= 1; o >>= 1) {
+        cost += __shfl_xor_sync(0xffffffffu, cost, o);
+        npos += __shfl_xor_sync(0xffffffffu, npos, o);
     }
-    __syncthreads();  // red is reused
-    if (lane == 0)
-#pragma unroll
-        for (int i = 0; i < N; ++i) red[i * kWarpsG + warp] = (double)x[i];
+    // bit 4 of the lane chose the upper eight values, bit 3 the upper four of those, ...
+    const int i = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
+    if (!(lane & 1)) S.part[warp][i] = v[0];
+    if (lane == 0) S.part[warp][16] = cost;
+    if (lane == 1) S.part[warp][17] = npos;
+}
+
+// Block sums in FP64 of the warp sums: warps 0..4 take four sums each, eight
+// lanes per sum.  Ends with a barrier; S.tot holds them.
+__device__ __forceinline__ void block_sums(Shared& S)
+{
+    static_assert(kWarpsG == 16, "eight lanes per sum add two warps each");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __syncthreads();
-    if (warp == 0) {
+    if (warp < (kSums + 3) / 4) {
+        const int i = warp * 4 + (lane >> 3), w = lane & 7;
+        double y = 0.0;
+        if (i < kSums) y = (double)S.part[w][i] + (double)S.part[w + 8][i];
 #pragma unroll
-        for (int i = 0; i < N; ++i) {
-            double y = lane < kWarpsG ? red[i * kWarpsG + lane] : 0.0;
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
-            if (lane == 0) red[i * kWarpsG] = y;
-        }
+        for (int o = 4; o >= 1; o >>= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+        if (i < kSums && w == 0) S.tot[i] = y;
     }
     __syncthreads();
-#pragma unroll
-    for (int i = 0; i < N; ++i) tot[i] = red[i * kWarpsG];
 }
 
 // Eigenvector of the largest eigenvalue of a symmetric 4 x 4 matrix (cyclic
@@ -126,14 +170,6 @@ __device__ void jacobi4_max(float (&A)[4][4], float (&q)[4])
     for (int k = 0; k < 4; ++k) q[k] = qv[k] * nrm;
 }
 
-struct Shared {
-    double red[16 * kWarpsG];
-    float R[9];      // current rotation (FP32, for the residuals)
-    float tc[3];     // translation in the centred frame: b' = R a' + tc
-    double Rd[9];    // current rotation, FP64 copy for the output
-    double c0[6];    // unweighted centroids of a and b (FP64)
-};
-
 // Per-point state in dynamic shared memory (struct of arrays).
 struct Pts {
     float* ax;
@@ -142,73 +178,79 @@ struct Pts {
     float* bx;
     float* by;
     float* bz;
-    float* w;
-    float* r2;
 };
 
-// Weighted fit in the centred frame: moments of the weighted points, then
-// Horn's quaternion (thread 0).  Returns the total weight.
-__device__ double fit(const Pts& P, int n, Shared& S)
+__device__ __forceinline__ void add_moments(float (&v)[16], const Pts& P, int k, float wk)
 {
-    float v[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = 0.f;
-    for (int k = threadIdx.x; k < n; k += kThreads) {
-        const float wk = P.w[k];
-        const float ax = P.ax[k], ay = P.ay[k], az = P.az[k], bx = P.bx[k], by = P.by[k], bz = P.bz[k];
-        v[0] += wk;
-        v[1] += wk * ax;
-        v[2] += wk * ay;
-        v[3] += wk * az;
-        v[4] += wk * bx;
-        v[5] += wk * by;
-        v[6] += wk * bz;
-        v[7] += wk * ax * bx;
-        v[8] += wk * ax * by;
-        v[9] += wk * ax * bz;
-        v[10] += wk * ay * bx;
-        v[11] += wk * ay * by;
-        v[12] += wk * ay * bz;
-        v[13] += wk * az * bx;
-        v[14] += wk * az * by;
-        v[15] += wk * az * bz;
-    }
-    double tot[16];
-    block_sum<16>(v, S.red, tot);
-    if (threadIdx.x == 0) {
-        const double sw = tot[0] > 0.0 ? tot[0] : 1.0;
-        const double ca[3] = {tot[1] / sw, tot[2] / sw, tot[3] / sw};
-        const double cb[3] = {tot[4] / sw, tot[5] / sw, tot[6] / sw};
+    const float ax = P.ax[k], ay = P.ay[k], az = P.az[k], bx = P.bx[k], by = P.by[k], bz = P.bz[k];
+    v[0] += wk;
+    v[1] += wk * ax;
+    v[2] += wk * ay;
+    v[3] += wk * az;
+    v[4] += wk * bx;
+    v[5] += wk * by;
+    v[6] += wk * bz;
+    v[7] += wk * ax * bx;
+    v[8] += wk * ax * by;
+    v[9] += wk * ax * bz;
+    v[10] += wk * ay * bx;
+    v[11] += wk * ay * by;
+    v[12] += wk * ay * bz;
+    v[13] += wk * az * bx;
+    v[14] += wk * az * by;
+    v[15] += wk * az * bz;
+}
+
+// Weighted fit in the centred frame from the moments in S.tot: Horn's
+// quaternion, rotation and translation.  Warp 0 works, one lane per entry;
+// ends with a barrier.
+__device__ void fit(Shared& S)
+{
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < 32) {
+        const double sw = S.tot[0] > 0.0 ? S.tot[0] : 1.0;
+        if (lane < 6) S.ca[lane] = S.tot[1 + lane] / sw;
+        __syncwarp();
+        const int e = lane < 9 ? lane : 8, i = e / 3, j = e - 3 * i;
         // centred cross-covariance S_ij = sum w (a_i - ca_i)(b_j - cb_j)
-        double H[3][3];
+        const float h = (float)(S.tot[7 + e] - sw * S.ca[i] * S.ca[3 + j]);
+        if (lane < 9) S.H[lane] = h;
+        __syncwarp();
+        if (lane == 0) {
+            const float Sxx = S.H[0], Sxy = S.H[1], Sxz = S.H[2];
+            const float Syx = S.H[3], Syy = S.H[4], Syz = S.H[5];
+            const float Szx = S.H[6], Szy = S.H[7], Szz = S.H[8];
+            float N[4][4] = {{Sxx + Syy + Szz, Syz - Szy, Szx - Sxz, Sxy - Syx},
+                             {Syz - Szy, Sxx - Syy - Szz, Sxy + Syx, Szx + Sxz},
+                             {Szx - Sxz, Sxy + Syx, -Sxx + Syy - Szz, Syz + Szy},
+                             {Sxy - Syx, Szx + Sxz, Syz + Szy, -Sxx - Syy + Szz}};
+            float q[4];
+            jacobi4_max(N, q);
 #pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) H[i][j] = tot[7 + 3 * i + j] - sw * ca[i] * cb[j];
-        const float Sxx = (float)H[0][0], Sxy = (float)H[0][1], Sxz = (float)H[0][2];
-        const float Syx = (float)H[1][0], Syy = (float)H[1][1], Syz = (float)H[1][2];
-        const float Szx = (float)H[2][0], Szy = (float)H[2][1], Szz = (float)H[2][2];
-        float N[4][4] = {{Sxx + Syy + Szz, Syz - Szy, Szx - Sxz, Sxy - Syx},
-                         {Syz - Szy, Sxx - Syy - Szz, Sxy + Syx, Szx + Sxz},
-                         {Szx - Sxz, Sxy + Syx, -Sxx + Syy - Szz, Syz + Szy},
-                         {Sxy - Syx, Szx + Sxz, Syz + Szy, -Sxx - Syy + Szz}};
-        float q[4];
-        jacobi4_max(N, q);
-        const double q0 = q[0], qx = q[1], qy = q[2], qz = q[3];
-        const double Rm[9] = {q0 * q0 + qx * qx - qy * qy - qz * qz, 2 * (qx * qy - q0 * qz), 2 * (qx * qz + q0 * qy),
-                              2 * (qx * qy + q0 * qz), q0 * q0 - qx * qx + qy * qy - qz * qz, 2 * (qy * qz - q0 * qx),
-                              2 * (qx * qz - q0 * qy), 2 * (qy * qz + q0 * qx), q0 * q0 - qx * qx - qy * qy + qz * qz};
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            S.Rd[i] = Rm[i];
-            S.R[i] = (float)Rm[i];
+            for (int k = 0; k < 4; ++k) S.q[k] = q[k];
         }
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-            S.tc[i] = (float)(cb[i] - (Rm[3 * i] * ca[0] + Rm[3 * i + 1] * ca[1] + Rm[3 * i + 2] * ca[2]));
+        __syncwarp();
+        // R = (q0^2 - |v|^2) I + 2 v v^T + 2 q0 [v]x, one entry per lane
+        const double q0 = S.q[0], vi = S.q[1 + i], vj = S.q[1 + j];
+        double r;
+        if (i == j) {
+            const double va = S.q[1 + (i + 1) % 3], vb = S.q[1 + (i + 2) % 3];
+            r = q0 * q0 + vi * vi - va * va - vb * vb;
+        } else {
+            const double vk = S.q[1 + 3 - i - j];
+            const double turn = q0 * vk;
+            r = 2 * (vi * vj + ((j + 3 - i) % 3 == 1 ? -turn : turn));
+        }
+        if (lane < 9) {
+            S.Rd[lane] = r;
+            S.R[lane] = (float)r;
+        }
+        __syncwarp();
+        if (lane < 3)
+            S.tc[lane] = (float)(S.ca[3 + lane] - (S.Rd[3 * lane] * S.ca[0] + S.Rd[3 * lane + 1] * S.ca[1] +
+                                                   S.Rd[3 * lane + 2] * S.ca[2]));
     }
     __syncthreads();
-    return tot[0];
 }
 
 __device__ __forceinline__ float resid2(const Shared& S, float ax, float ay, float az, float bx, float by, float bz)
@@ -227,7 +269,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 {
     __shared__ Shared S;
     const int64_t n64 = d_n ? min(*d_n, cap) : cap;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (n64 > (int64_t)kMaxPoints) {  // more points than shared memory holds
         if (tid == 0) {
             kmx_raise(err, KMX_DERR_CAPACITY);
@@ -250,43 +292,47 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     extern __shared__ float dyn[];
     const Pts P{dyn, dyn + kMaxPoints, dyn + 2 * kMaxPoints, dyn + 3 * kMaxPoints, dyn + 4 * kMaxPoints,
-                dyn + 5 * kMaxPoints, dyn + 6 * kMaxPoints, dyn + 7 * kMaxPoints};
+                dyn + 5 * kMaxPoints};
+    float* w = dyn + 6 * kMaxPoints;       // the weights of the latest fit
+    float* w_next = dyn + 7 * kMaxPoints;  // the next ones
     // unweighted centroids in FP64, the reference frame of the FP32 work:
     // offsets from the first point are summed, then it is added back
     const kmx_corr c0 = corr[sel[inlier[0]]];
     const float4 a0 = src4[c0.i], b0 = tgt4[c0.j];
-    {
-        float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int k = tid; k < n; k += kThreads) {
-            const kmx_corr c = corr[sel[inlier[k]]];
-            const float4 a = src4[c.i], b = tgt4[c.j];
-            P.ax[k] = a.x;  // raw for now, centred below
-            P.ay[k] = a.y;
-            P.az[k] = a.z;
-            P.bx[k] = b.x;
-            P.by[k] = b.y;
-            P.bz[k] = b.z;
-            v[0] += a.x - a0.x;
-            v[1] += a.y - a0.y;
-            v[2] += a.z - a0.z;
-            v[3] += b.x - b0.x;
-            v[4] += b.y - b0.y;
-            v[5] += b.z - b0.z;
-        }
-        double tot[6];
-        block_sum<6>(v, S.red, tot);
-        if (tid == 0) {
-            S.c0[0] = (double)a0.x + tot[0] / n;
-            S.c0[1] = (double)a0.y + tot[1] / n;
-            S.c0[2] = (double)a0.z + tot[2] / n;
-            S.c0[3] = (double)b0.x + tot[3] / n;
-            S.c0[4] = (double)b0.y + tot[4] / n;
-            S.c0[5] = (double)b0.z + tot[5] / n;
-        }
-        __syncthreads();
+    float v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = 0.f;
+    for (int k = tid; k < n; k += kThreads) {
+        const kmx_corr c = corr[sel[inlier[k]]];
+        const float4 a = src4[c.i], b = tgt4[c.j];
+        P.ax[k] = a.x;  // raw for now, centred below
+        P.ay[k] = a.y;
+        P.az[k] = a.z;
+        P.bx[k] = b.x;
+        P.by[k] = b.y;
+        P.bz[k] = b.z;
+        v[0] += a.x - a0.x;
+        v[1] += a.y - a0.y;
+        v[2] += a.z - a0.z;
+        v[3] += b.x - b0.x;
+        v[4] += b.y - b0.y;
+        v[5] += b.z - b0.z;
     }
-    const double ca0[3] = {S.c0[0], S.c0[1], S.c0[2]};
-    const double cb0[3] = {S.c0[3], S.c0[4], S.c0[5]};
+    warp_sums(v, 0.f, 0.f, S);
+    block_sums(S);
+    double ca0[3], cb0[3];
+    {
+        const float first[6] = {a0.x, a0.y, a0.z, b0.x, b0.y, b0.z};
+        if (tid < 6) S.ca[tid] = (double)first[tid] + S.tot[tid] / n;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            ca0[i] = S.ca[i];
+            cb0[i] = S.ca[3 + i];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = 0.f;
     for (int k = tid; k < n; k += kThreads) {
         P.ax[k] = (float)((double)P.ax[k] - ca0[0]);
         P.ay[k] = (float)((double)P.ay[k] - ca0[1]);
@@ -294,74 +340,87 @@ __global__ void __launch_bounds__(kThreads, 1)
         P.bx[k] = (float)((double)P.bx[k] - cb0[0]);
         P.by[k] = (float)((double)P.by[k] - cb0[1]);
         P.bz[k] = (float)((double)P.bz[k] - cb0[2]);
-        P.w[k] = 1.f;
+        w[k] = 1.f;
+        add_moments(v, P, k, 1.f);
     }
-    __syncthreads();
-    fit(P, n, S);
+    warp_sums(v, 0.f, 0.f, S);
+    block_sums(S);
+    fit(S);
     float rmax = 0.f;
-    for (int k = tid; k < n; k += kThreads) {
-        const float r = resid2(S, P.ax[k], P.ay[k], P.az[k], P.bx[k], P.by[k], P.bz[k]);
-        P.r2[k] = r;
-        rmax = fmaxf(rmax, r);
-    }
+    for (int k = tid; k < n; k += kThreads)
+        rmax = fmaxf(rmax, resid2(S, P.ax[k], P.ay[k], P.az[k], P.bx[k], P.by[k], P.bz[k]));
     {
-#pragma unroll
-        for (int sh = 16; sh >= 1; sh >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, sh));
+        // residuals are >= 0 (or NaN, which fmaxf drops): their bits order like integers
+        const unsigned wm = __reduce_max_sync(0xffffffffu, __float_as_uint(rmax));
+        if (lane == 0) S.count[warp] = (int32_t)wm;
         __syncthreads();
-        if ((tid & 31) == 0) S.red[tid >> 5] = rmax;
-        __syncthreads();
-        double m = 0.0;
-        for (int i = 0; i < kWarpsG; ++i) m = fmax(m, S.red[i]);
-        rmax = (float)m;
+        rmax = __uint_as_float(__reduce_max_sync(0xffffffffu, (unsigned)S.count[lane % kWarpsG]));
         __syncthreads();
     }
     int iters = 0;
     if ((double)rmax > c2) {
-        double mu = c2 / fmax(2.0 * (double)rmax - c2, 1e-30);
+        double mu0 = c2 / fmax(2.0 * (double)rmax - c2, 1e-30);  // of the schedule's first entry
         double prev_cost = INFINITY;
         for (int it = 0; it < max_iters; ++it) {
-            const float lo = (float)(mu / (mu + 1.0) * c2), hi = (float)((mu + 1.0) / mu * c2);
-            const float cw = (float)(sqrt(c2) * sqrt(mu * (mu + 1.0))), muf = (float)mu;
-            float npos[1] = {0.f};
-            for (int k = tid; k < n; k += kThreads) {
-                const float r = P.r2[k];
-                const float wk = r <= lo ? 1.f : (r >= hi ? 0.f : cw / sqrtf(fmaxf(r, 1e-30f)) - muf);
-                P.w[k] = wk;
-                npos[0] += wk > 0.f ? 1.f : 0.f;
+            if ((it & 31) == 0) {
+                // the schedule of 32 iterations, by as many lanes (every warp
+                // has passed the last barrier, so the last entries are read)
+                if (warp == 0) {
+                    double mu = mu0;
+                    for (int i = 0; i < lane; ++i) mu *= mu_factor;
+                    S.sched[lane] = make_float4((float)(mu / (mu + 1.0) * c2), (float)((mu + 1.0) / mu * c2),
+                                                (float)(sqrt(c2) * sqrt(mu * (mu + 1.0))), (float)mu);
+                    mu0 = __shfl_sync(0xffffffffu, mu, 31) * mu_factor;
+                }
+                __syncthreads();
             }
-            double ctot[1];
-            block_sum<1>(npos, S.red, ctot);
-            if (ctot[0] < 3.0) break;  // the current fit stays; w are the weights that stopped it
-            fit(P, n, S);
-            ++iters;
-            float cv[1] = {0.f};
+            // residuals of the last fit, its cost, and the next weights with
+            // their moments
+            const float4 sc = S.sched[it & 31];
+            float cost = 0.f, npos = 0.f;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = 0.f;
             for (int k = tid; k < n; k += kThreads) {
                 const float r = resid2(S, P.ax[k], P.ay[k], P.az[k], P.bx[k], P.by[k], P.bz[k]);
-                P.r2[k] = r;
-                cv[0] += P.w[k] * r;
+                cost += w[k] * r;
+                const float wk = r <= sc.x ? 1.f : (r >= sc.y ? 0.f : sc.z / sqrtf(fmaxf(r, 1e-30f)) - sc.w);
+                w_next[k] = wk;
+                npos += wk > 0.f ? 1.f : 0.f;
+                add_moments(v, P, k, wk);
             }
-            double cost[1];
-            block_sum<1>(cv, S.red, cost);
-            if (fabs(cost[0] - prev_cost) < tol) break;
-            prev_cost = cost[0];
-            mu *= mu_factor;
+            warp_sums(v, cost, npos, S);
+            block_sums(S);
+            if (it > 0) {
+                if (fabs(S.tot[16] - prev_cost) < tol) break;
+                prev_cost = S.tot[16];
+            }
+            float* const t = w;
+            w = w_next;
+            w_next = t;
+            if (S.tot[17] < 3.0) break;  // the current fit stays; w are the weights that stopped it
+            fit(S);
+            ++iters;
         }
     }
     // outputs: R, t in the original frame (b = R a + t with t = cb0 + tc - R ca0)
-    float good[1] = {0.f};
+    int good = 0;
     for (int k = tid; k < n; k += kThreads) {
-        o.w[k] = P.w[k];
-        good[0] += P.w[k] > 0.5f ? 1.f : 0.f;
+        const float wk = w[k];
+        o.w[k] = wk;
+        good += wk > 0.5f;
     }
-    double gt[1];
-    block_sum<1>(good, S.red, gt);
+    good = __reduce_add_sync(0xffffffffu, good);
+    if (lane == 0) S.count[warp] = good;
+    __syncthreads();
     if (tid == 0) {
         for (int i = 0; i < 9; ++i) o.R[i] = S.Rd[i];
         for (int i = 0; i < 3; ++i)
             o.t[i] = cb0[i] + (double)S.tc[i] -
                      (S.Rd[3 * i] * ca0[0] + S.Rd[3 * i + 1] * ca0[1] + S.Rd[3 * i + 2] * ca0[2]);
         o.stats[0] = iters;
-        o.stats[1] = (int32_t)gt[0];
+        good = 0;
+        for (int i = 0; i < kWarpsG; ++i) good += S.count[i];
+        o.stats[1] = good;
         o.stats[2] = n;
         o.stats[3] = 0;
     }
