@@ -39,7 +39,7 @@
 //             (triangle inequality; tested first for the whole row tile with
 //             the largest |x - c_R| + sqrt(U) around its own centre c_R, then
 //             row by row, with margins for FP32 rounding).  The tiles that pass form the row tile's list,
-//             cut into work items of 32 tiles.
+//             cut into work items of 8 to 32 tiles.
 //   collect   persistent CTAs (two per SM), each taking every gridDim-th work item: per
 //             column tile of the item the CTA writes its row tile re-centred
 //             on the column tile's centre as the A operand
@@ -121,9 +121,13 @@ constexpr int kColBytes = kHdrGBeta + (kTN / 8) * 4;  // 13024, a multiple of 16
 constexpr int kStages = 4;                    // column-tile ring
 constexpr int kThreads = 320;                 // 10 warps (roles in tc_collect)
 constexpr int kCtasPerSm = 2;                 // of tc_collect
+constexpr int kListCtas = 7;                  // of tc_lists per SM (registers)
 constexpr int kTmemCols = 256;                // two 128-column FP32 accumulators per CTA
 constexpr int kCandCap = 512;                 // candidate list per row
-constexpr int kItemTiles = 32;                // column tiles per work item (a power of two)
+constexpr int kItemTiles = 32;                // column tiles per work item, at most
+constexpr int kItemMin = 8;                   // and at least, but for the last of a list
+constexpr int kItemsPerCta = 6;               // wanted, as far as kItemMin allows
+constexpr int kListSeg = 32;                  // column tiles, the unit by which a row tile's list is cut among CTAs
 constexpr int kPlanRec = 32;                  // columns of the nearest tile recorded per row in the plan
 constexpr int kCandBuf = 16;                  // candidates buffered per row in the collect kernel
 constexpr float kC = 0.008f;                  // c' of the bounds
@@ -1011,12 +1015,9 @@ __device__ __forceinline__ bool tile_may_hold(float dist, float rad, float u2)
     return !(g > 0.f && g * g * (1.f - kTolD) > u2);
 }
 
-// A work item: a row tile, the first of its list's column tiles (a multiple of
-// kItemTiles) and, in the low bits, how many tiles less one.
-__device__ __forceinline__ int2 pack_item(int rt, int first, int total)
-{
-    return make_int2(rt, first | (min(kItemTiles, total - first) - 1));
-}
+// A work item: a row tile (24 bits, tiles of at most 2^31 rows), how many column
+// tiles less one (above), and the place of the first in the row tile's list.
+__device__ __forceinline__ int2 pack_item(int rt, int first, int n) { return make_int2(rt | (n - 1) << 24, first); }
 
 // Shared memory of a plan CTA.
 struct PlanShared {
@@ -1030,6 +1031,7 @@ struct PlanShared {
     int wcnt[kTN / 32];
     float redf[kTN / 32];
     int redi[kTN / 32];
+    float mean[kTN / 32][kCenterStride];
     int cs, total, next;
 };
 
@@ -1050,6 +1052,7 @@ struct PlanDir {
     float* ub;
     int32_t* need;
     int64_t need_stride;
+    int32_t* near;  // the nearest column tile of each row tile (tc_near)
     int32_t* nneed;
     int2* items;
     int* n_items;
@@ -1077,10 +1080,11 @@ __device__ __forceinline__ void load_row(const float* __restrict__ row, bool val
 //      path's arithmetic): its second-smallest d2 over distinct columns is
 //      an upper bound of the row's d(2); the columns with distance <= d2
 //      are its first candidates (cnt[row] = their number), and ub[row] = d2.
-// Returns d2; x is the row, cR (shared) its tile's centre and S.cs the tile.
-__device__ __forceinline__ float plan_nearest(PlanShared& S, const PlanDir& D, const int64_t rt, const int64_t rows,
-                                              const int64_t cols, float (&x)[KMX_DESC_DIM])
+// near[rt] is the tile cs.
+__device__ __forceinline__ void plan_nearest(PlanShared& S, const PlanDir& D, const int64_t rt, const int64_t rows,
+                                             const int64_t cols)
 {
+    float x[KMX_DESC_DIM];
     float(*ys)[kCenterStride] = S.ysc;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t n_ct = (cols + kTN - 1) / kTN;
@@ -1123,6 +1127,7 @@ __device__ __forceinline__ float plan_nearest(PlanShared& S, const PlanDir& D, c
                     i0 = S.redi[q];
                 }
             S.cs = i0 == 0x7fffffff ? 0 : i0;
+            D.near[rt] = S.cs;
         }
         __syncthreads();
     }
@@ -1220,23 +1225,22 @@ __device__ __forceinline__ float plan_nearest(PlanShared& S, const PlanDir& D, c
         D.cnt[xrow] = k;
         D.ub[xrow] = d2;
     }
-    return d2;
 }
 
-// The column tiles other than `skip` that tile_may_hold for some
-// row of the CTA, in increasing order, into need[rt * need_stride ...];
-// nneed[rt] = their number, and the list is cut into items of kItemTiles tiles
-// appended to `items`.  x is the thread's row, U the squared distance within
-// which it needs columns (negative: none), S.cR a centre near the CTA's rows.
-// A row reaches a tile with centre c and radius r only if |cR - c| - r <=
+// The column tiles u0 .. u1 - 1 other than `skip` that tile_may_hold for some
+// row of the CTA, in increasing order, into need[rt * need_stride + u0 ...];
+// their number is added to nneed[rt], and they are cut into items of item_len
+// tiles appended to `items`.  x is the thread's row, U the squared distance
+// within which it needs columns (negative: none), S.cR a centre near the CTA's
+// rows.  A row reaches a tile with centre c and radius r only if |cR - c| - r <=
 // |x - cR| + sqrt(U): the largest right side over the rows decides first, for
 // all rows at once, which tiles are tested row by row.
-__device__ __forceinline__ void plan_list(PlanShared& S, const PlanDir& D, const int64_t rt, const int64_t cols,
-                                          const int64_t skip, const float (&x)[KMX_DESC_DIM], const float U)
+__device__ __forceinline__ void plan_list(PlanShared& S, const PlanDir& D, const int64_t rt, const int64_t u0,
+                                          const int64_t u1, const int64_t skip, const int item_len,
+                                          const float (&x)[KMX_DESC_DIM], const float U)
 {
     float(*sc)[kCenterStride] = S.ysc;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t n_ct = (cols + kTN - 1) / kTN;
     float reach = -1.f;
     if (U >= 0.f) {
         float e2 = 0.f;
@@ -1257,13 +1261,13 @@ __device__ __forceinline__ void plan_list(PlanShared& S, const PlanDir& D, const
 #pragma unroll
     for (int h = 0; h < KMX_DESC_DIM; ++h) xx = fmaf(x[h], x[h], xx);
     const float xn = sqrtf(xx);
-    // 3. the other column tiles, 128 at a time
+    // 128 column tiles at a time
     const bool busy = __any_sync(0xffffffffu, U >= 0.f);  // the warp has a row to test
-    for (int64_t base = 0; base < n_ct; base += kTN) {
+    for (int64_t base = u0; base < u1; base += kTN) {
         const int64_t u = base + tid;
         bool surv = false;
         float ru = 0.f;
-        if (u < n_ct && u != skip) {
+        if (u < u1 && u != skip) {
             const float* c = D.cenY + u * kCenterStride;
             const float d = centre_dist2(S.cR, c);
             ru = sqrtf(__ldg(c + KMX_DESC_DIM));
@@ -1352,7 +1356,7 @@ __device__ __forceinline__ void plan_list(PlanShared& S, const PlanDir& D, const
             if ((word >> (tid & 31)) & 1u) {
                 int rank = __popc(word & ((1u << (tid & 31)) - 1u));
                 for (int q = 0; q < (tid >> 5); ++q) rank += __popc(S.needbits[q]);
-                D.need[rt * D.need_stride + S.total + rank] = S.sid[tid];
+                D.need[rt * D.need_stride + u0 + S.total + rank] = S.sid[tid];
             }
         }
         __syncthreads();
@@ -1362,21 +1366,20 @@ __device__ __forceinline__ void plan_list(PlanShared& S, const PlanDir& D, const
     }
     if (tid == 0) {
         const int total = S.total;
-        D.nneed[rt] = total;
-        const int nit = (total + kItemTiles - 1) / kItemTiles;
+        const int nit = (total + item_len - 1) / item_len;
         if (nit > 0) {
+            atomicAdd(D.nneed + rt, total);
             const int b = atomicAdd(D.n_items, nit);
-            for (int i = 0; i < nit; ++i) D.items[b + i] = pack_item((int)rt, i * kItemTiles, total);
+            for (int i = 0; i < nit; ++i)
+                D.items[b + i] = pack_item((int)rt, (int)u0 + i * item_len, min(item_len, total - i * item_len));
         }
     }
 }
 
-// Both directions in one launch (one tail instead of two): CTAs take row
-// tiles from a counter (*next, zeroed before the launch).  Source row tiles
-// (a) get their first candidates, bounds and tile lists; target row tiles (b)
-// only the first two, since their lists wait for the source rows' results
-// (tc_plan_back).
-__global__ void __launch_bounds__(kTM) tc_plan(PlanDir a, PlanDir b, int* __restrict__ next)
+// First candidates and bounds of both sides' rows in one launch (one tail
+// instead of two): CTAs take row tiles from a counter (*next, zeroed before the
+// launch), first those of direction a, then those of b.
+__global__ void __launch_bounds__(kTM) tc_near(PlanDir a, PlanDir b, int* __restrict__ next)
 {
     __shared__ PlanShared S;
     const int64_t na = kmx_count(a.d_nx, a.nx_cap), nb = kmx_count(b.d_nx, b.nx_cap);
@@ -1388,15 +1391,74 @@ __global__ void __launch_bounds__(kTM) tc_plan(PlanDir a, PlanDir b, int* __rest
         const int64_t k = S.next;
         __syncthreads();  // S.next is read before thread 0 takes the next tile
         if (k >= ta + tb) break;
-        float x[KMX_DESC_DIM];
-        if (k < ta) {
-            const float d2 = plan_nearest(S, a, k, na, nb, x);
-            __syncthreads();  // the shared rows become the tile list's centres
-            plan_list(S, a, k, nb, S.cs, x, k * kTM + threadIdx.x < na ? d2 : -1.f);
-        } else {
-            plan_nearest(S, b, k - ta, nb, na, x);
-        }
+        if (k < ta)
+            plan_nearest(S, a, k, na, nb);
+        else
+            plan_nearest(S, b, k - ta, nb, na);
         __syncthreads();  // the next tile rewrites the shared arrays
+    }
+}
+
+// Column tile lists of the rows of direction d.  Source side (kBack false): all
+// row tiles, each without its nearest column tile.  Target side: the rows
+// `rows` (positions in tree order, *n_rows of them, 128 to a row tile; their
+// order is the tree's, so a tile's rows are near each other), with every column
+// tile, since a row tile's rows come from several leaves, each with a nearest
+// one of its own.  A unit of work is one row tile against a part of the column
+// tiles, in as many parts as give every CTA about four units: whole lists on
+// large clouds (long items for tc_collect), parts where row tiles are few.
+// Whole lists, formed after the nearest tile by the same CTA, and items of 32
+// tiles left most SMs idle on small clouds: at 40009 x 61003 rows plan and
+// collect took 151 + 155 us (source side) and 80 + 46 us (target side), now 91
+// (tc_near, both sides) + 38 + 116 us and 16 + 23 us; at 302548 x 287858 rows
+// the whole match went from 4.45 to 4.03 ms.
+template <bool kBack>
+__global__ void __launch_bounds__(kTM, kListCtas) tc_lists(PlanDir d, const int32_t* __restrict__ rows,
+                                                const int64_t* __restrict__ n_rows, int collect_ctas,
+                                                int* __restrict__ next)
+{
+    __shared__ PlanShared S;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t n = kBack ? *n_rows : kmx_count(d.d_nx, d.nx_cap), ny = kmx_count(d.d_ny, d.ny_cap);
+    if (n <= 0 || ny <= 0) return;
+    const int64_t tiles = (n + kTM - 1) / kTM, n_ct = (ny + kTN - 1) / kTN;
+    const int64_t segs = (n_ct + kListSeg - 1) / kListSeg;
+    const int64_t want = min(segs, (4 * (int64_t)gridDim.x + tiles - 1) / tiles);
+    const int64_t part = (segs + want - 1) / want, parts = (segs + part - 1) / part;
+    // items for kItemsPerCta rounds of tc_collect if a twelfth of the pairs is kept
+    const int item_len = (int)min((int64_t)kItemTiles,
+                                  max((int64_t)kItemMin, tiles * n_ct / (12 * kItemsPerCta * (int64_t)collect_ctas)));
+    for (;;) {
+        if (tid == 0) S.next = atomicAdd(next, 1);
+        __syncthreads();
+        const int64_t k = S.next;
+        __syncthreads();
+        if (k >= tiles * parts) break;
+        const int64_t rt = k / parts, u0 = (k - rt * parts) * part * kListSeg;
+        const int64_t i = rt * kTM + tid;
+        const bool valid = i < n;
+        const int64_t pos = valid ? (kBack ? (int64_t)rows[i] : i) : 0;
+        float x[KMX_DESC_DIM];
+        load_row(d.X + (valid ? (int64_t)d.permX[pos] * KMX_DESC_STRIDE : 0), valid, x);
+        if (kBack) {  // the rows' own mean: they may come from far more than one leaf
+#pragma unroll
+            for (int h = 0; h < KMX_DESC_DIM; ++h) {
+                float m = x[h];
+#pragma unroll
+                for (int o = 16; o >= 1; o >>= 1) m += __shfl_xor_sync(0xffffffffu, m, o);
+                if (lane == 0) S.mean[warp][h] = m;
+            }
+            __syncthreads();
+            if (tid < KMX_DESC_DIM)
+                S.cR[tid] = (S.mean[0][tid] + S.mean[1][tid] + S.mean[2][tid] + S.mean[3][tid]) /
+                            (float)min((int64_t)kTM, n - rt * kTM);
+        } else if (tid < KMX_DESC_DIM) {
+            S.cR[tid] = d.cenX[rt * kCenterStride + tid];
+        }
+        __syncthreads();
+        plan_list(S, d, rt, u0, min(n_ct, u0 + part * kListSeg), kBack ? -1 : (int64_t)d.near[rt], item_len, x,
+                  valid ? d.ub[pos] : -1.f);
+        __syncthreads();
     }
 }
 
@@ -1427,41 +1489,6 @@ __global__ void __launch_bounds__(256) back_rows(const int32_t* __restrict__ per
         if (!flag[i]) continue;
         ub[i] = fminf(ub[i], __uint_as_float((uint32_t)(colbest[permQ[i]] >> 32)));
         rows[pos[i]] = (int32_t)i;
-    }
-}
-
-// Tile lists of the target rows `rows` (positions in tree order, *n_rows of
-// them, 128 to a row tile; their order is the tree's, so a tile's rows are near
-// each other).  The plan's nearest column tile is listed again: a row tile's rows
-// come from several leaves, each with its own.
-__global__ void __launch_bounds__(kTM) tc_plan_back(PlanDir d, const int32_t* __restrict__ rows,
-                                                    const int64_t* __restrict__ n_rows, int* __restrict__ next)
-{
-    __shared__ PlanShared S;
-    const int tid = threadIdx.x;
-    const int64_t n = *n_rows, nx = kmx_count(d.d_nx, d.nx_cap), ny = kmx_count(d.d_ny, d.ny_cap);
-    const int64_t tiles = (n + kTM - 1) / kTM, all = (nx + kTM - 1) / kTM;
-    if (nx <= 0 || ny <= 0) return;
-    for (;;) {
-        if (tid == 0) S.next = atomicAdd(next, 1);
-        __syncthreads();
-        const int64_t k = S.next;
-        __syncthreads();
-        if (k >= all) break;
-        if (k >= tiles) {
-            if (tid == 0) d.nneed[k] = 0;
-            continue;
-        }
-        const int64_t i = k * kTM + tid;
-        const bool valid = i < n;
-        const int32_t pos = valid ? rows[i] : 0;
-        float x[KMX_DESC_DIM];
-        load_row(d.X + (valid ? (int64_t)d.permX[pos] * KMX_DESC_STRIDE : 0), valid, x);
-        const int64_t mid = rows[min(k * kTM + kTM / 2, n - 1)] / kTM;
-        if (tid < KMX_DESC_DIM) S.cR[tid] = d.cenX[mid * kCenterStride + tid];
-        __syncthreads();
-        plan_list(S, d, k, ny, -1, x, valid ? d.ub[pos] : -1.f);
-        __syncthreads();
     }
 }
 
@@ -1540,9 +1567,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) tc_collect(const float* 
     if ((int)blockIdx.x >= nit) return;
     const int stride = (int)gridDim.x;
     auto item_tiles = [&](int2 item, const int32_t*& tl, int64_t& rt) -> int {
-        rt = item.x;
-        tl = need + (int64_t)item.x * need_stride + (item.y & ~(kItemTiles - 1));
-        return (item.y & (kItemTiles - 1)) + 1;
+        rt = item.x & 0xffffff;
+        tl = need + rt * need_stride + item.y;
+        return (item.x >> 24) + 1;
     };
     // position of a row in tree order (the index of its bound and candidates)
     auto position = [&](int64_t i) -> int64_t { return kBack ? (int64_t)rowmap[i] : i; };
@@ -1725,7 +1752,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) tc_collect(const float* 
         bool dead = false;
         int2 item = item_at(blockIdx.x);
         int64_t next_row = 0;
-        float Unext = bound_at(item.x, next_row);
+        float Unext = bound_at(item.x & 0xffffff, next_row);
         for (int it = blockIdx.x; it < nit && !dead; it += stride) {
             const int32_t* tl;
             int64_t rt;
@@ -1741,7 +1768,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) tc_collect(const float* 
             for (int k = 0; k < nt; ++k, ++t) {
                 const int sa = t % kAStages, ab = t % kAccBufs;
                 const int tile = tl[k];
-                if (k + 1 == nt) Unext = bound_at(item.x, next_row);
+                if (k + 1 == nt) Unext = bound_at(item.x & 0xffffff, next_row);
                 bool ok = !*failed;
                 if (ok) ok = mbar_wait(&S.acc_full[ab], (t / kAccBufs) & 1);
                 // the A stage (row constants) cannot be refilled before these
@@ -2004,15 +2031,16 @@ struct TcBuffers {
     uint8_t *packP, *packQ;
     float *cenP, *cenQ;
     float *ubP, *ubQ;
-    int32_t *needP, *needQ, *nneedP, *nneedQ;
+    int32_t *needP, *needQ, *nneedP, *nneedQ, *nearP, *nearQ;
     int2 *itemsP, *itemsQ;
-    int* nitems;               // [0] source rows, [1] target rows, [2], [3] the plans' tile counters
+    int* nitems;               // [0] source rows, [1] target rows, [2] .. [4] work counters of tc_near and tc_lists
     int32_t *flag, *rowsQ;     // target rows that are some source row's nearest: flags, then their positions
     int64_t* flagpos;          // scanned flags; [nq_cap] = how many
     int32_t *candP, *candQ, *cntP, *cntQ;
     int* chunks;               // [2] fallback P, [3] fallback Q
     int32_t *listP, *listQ;    // fallback rows (original indices)
     int64_t* nlist;            // their counts: [0] P, [1] Q
+    size_t zeroed;             // bytes from nlist on that are zeroed before each match
     kmx::RowBest *fbP, *fbQ;
 };
 
@@ -2048,22 +2076,29 @@ TcBuffers tc_carve(void* base, int64_t np_cap, int64_t nq_cap, size_t* total)
     b.ubQ = (float*)a.take(sizeof(float) * (size_t)nq_cap);
     b.needP = (int32_t*)a.take(sizeof(int32_t) * (size_t)tp * (size_t)tq);
     b.needQ = (int32_t*)a.take(sizeof(int32_t) * (size_t)tq * (size_t)tp);
-    b.nneedP = (int32_t*)a.take(sizeof(int32_t) * (size_t)tp);
-    b.nneedQ = (int32_t*)a.take(sizeof(int32_t) * (size_t)tq);
-    b.itemsP = (int2*)a.take(sizeof(int2) * (size_t)tp * (size_t)((tq + kItemTiles - 1) / kItemTiles));
-    b.itemsQ = (int2*)a.take(sizeof(int2) * (size_t)tq * (size_t)((tp + kItemTiles - 1) / kItemTiles));
-    b.nitems = (int*)a.take(sizeof(int) * 4);
+    b.nearP = (int32_t*)a.take(sizeof(int32_t) * (size_t)(tp + tq));
+    b.nearQ = b.nearP + tp;
+    // a list is cut into items of kItemMin or more, but for one at the end of each part
+    const int64_t ip = (tq + kItemMin - 1) / kItemMin + (tq + kListSeg - 1) / kListSeg;
+    const int64_t iq = (tp + kItemMin - 1) / kItemMin + (tp + kListSeg - 1) / kListSeg;
+    b.itemsP = (int2*)a.take(sizeof(int2) * (size_t)tp * (size_t)ip);
+    b.itemsQ = (int2*)a.take(sizeof(int2) * (size_t)tq * (size_t)iq);
+    // zeroed together: fallback counts, item and work counters, list lengths, candidate counts
+    b.zeroed = (size_t)(sizeof(int64_t) * 2 + sizeof(int) * 6) + sizeof(int32_t) * (size_t)(tp + tq + n2);
+    b.nlist = (int64_t*)a.take(b.zeroed);
+    b.nitems = (int*)(b.nlist + 2);
+    b.nneedP = b.nitems + 6;
+    b.nneedQ = b.nneedP + tp;
+    b.cntP = b.nneedQ + tq;
+    b.cntQ = b.cntP + np_cap;
     b.flag = (int32_t*)b.keys;      // the tree's keys and entries are no longer needed then
     b.rowsQ = b.vals_tmp;
     b.flagpos = (int64_t*)a.take(sizeof(int64_t) * (size_t)(nq_cap + 1));
     b.candP = (int32_t*)a.take(sizeof(int32_t) * kCandCap * (size_t)np_cap);
     b.candQ = (int32_t*)a.take(sizeof(int32_t) * kCandCap * (size_t)nq_cap);
-    b.cntP = (int32_t*)a.take(sizeof(int32_t) * (size_t)(np_cap + nq_cap));
-    b.cntQ = b.cntP + np_cap;
     b.chunks = (int*)a.take(sizeof(int) * 4);
     b.listP = (int32_t*)a.take(sizeof(int32_t) * (np_cap + 1));
     b.listQ = (int32_t*)a.take(sizeof(int32_t) * (nq_cap + 1));
-    b.nlist = (int64_t*)a.take(sizeof(int64_t) * 2);
     b.fbP = (kmx::RowBest*)a.take(sizeof(kmx::RowBest) * (size_t)fc * (np_cap + 1));
     b.fbQ = (kmx::RowBest*)a.take(sizeof(kmx::RowBest) * (size_t)fc * (nq_cap + 1));
     *total = kmx_align_up(a.used, 256);
@@ -2107,9 +2142,7 @@ cudaError_t kmx_match_tc_launch(kmx_ctx* ctx, const float* dp, int64_t np_cap, c
         return cudaFuncSetAttribute(tree_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFinishSmem);
     });
     if (e) return e;
-    if ((e = cudaMemsetAsync(b.nlist, 0, sizeof(int64_t) * 2, st))) return e;
-    if ((e = cudaMemsetAsync(b.cntP, 0, sizeof(int32_t) * (size_t)n2, st))) return e;
-    if ((e = cudaMemsetAsync(b.nitems, 0, sizeof(int) * 4, st))) return e;
+    if ((e = cudaMemsetAsync(b.nlist, 0, b.zeroed, st))) return e;
     // locality order of both clouds: one tree level per sort
     const unsigned gb = kmx_stride_blocks(n2, 256, ctx->sm_count);
     KMX_COUNT_LAUNCH();
@@ -2169,17 +2202,20 @@ cudaError_t kmx_match_tc_launch(kmx_ctx* ctx, const float* dp, int64_t np_cap, c
     KMX_COUNT_LAUNCH();
     tc_pack<<<kmx_stride_blocks(tq, 1, ctx->sm_count, 16), kTN, 0, st>>>(dq, permQ, nq_cap, d_nq, b.packQ, b.cenQ,
                                                                         ctx->d_err);
-    // first candidates, bounds and tile lists both ways
+    // first candidates and bounds both ways, the source rows' tile lists
     const PlanDir planP{dp, permP, np_cap, d_np, b.cenP, dq, permQ, nq_cap, d_nq, b.cenQ, b.candP,
-                        b.cntP, b.ubP, b.needP, tq, b.nneedP, b.itemsP, b.nitems + 0};
+                        b.cntP, b.ubP, b.needP, tq, b.nearP, b.nneedP, b.itemsP, b.nitems + 0};
     const PlanDir planQ{dq, permQ, nq_cap, d_nq, b.cenQ, dp, permP, np_cap, d_np, b.cenP, b.candQ,
-                        b.cntQ, b.ubQ, b.needQ, tp, b.nneedQ, b.itemsQ, b.nitems + 1};
+                        b.cntQ, b.ubQ, b.needQ, tp, b.nearQ, b.nneedQ, b.itemsQ, b.nitems + 1};
     KMX_COUNT_LAUNCH();
     // about five CTAs per SM fit (registers); more would only wait for the counter
-    tc_plan<<<kmx_stride_blocks(tp + tq, 1, ctx->sm_count, 5), kTM, 0, st>>>(planP, planQ, b.nitems + 2);
+    tc_near<<<kmx_stride_blocks(tp + tq, 1, ctx->sm_count, 5), kTM, 0, st>>>(planP, planQ, b.nitems + 2);
+    const unsigned sms = (unsigned)(ctx->sm_count > 0 ? ctx->sm_count : 1);
+    const unsigned grid = kCtasPerSm * sms;  // of tc_collect: persistent CTAs
+    KMX_COUNT_LAUNCH();
+    tc_lists<false><<<kListCtas * sms, kTM, 0, st>>>(planP, nullptr, nullptr, (int)grid, b.nitems + 3);
     // source rows: tensor-core candidates (persistent CTAs), exact re-ranking,
     // exact fallback for the overflowed rows
-    const unsigned grid = (unsigned)(ctx->sm_count > 0 ? kCtasPerSm * ctx->sm_count : 1);
     KMX_COUNT_LAUNCH();
     tc_collect<false><<<grid, kThreads, smem, st>>>(dp, permP, np_cap, d_np, nullptr, b.packQ, b.needP, tq, b.itemsP,
                                                     b.nitems + 0, b.ubP, b.candP, b.cntP, ctx->d_err);
@@ -2204,8 +2240,7 @@ cudaError_t kmx_match_tc_launch(kmx_ctx* ctx, const float* dp, int64_t np_cap, c
     KMX_COUNT_LAUNCH();
     back_rows<<<qb, 256, 0, st>>>(permQ, nq_cap, d_nq, s.colbest, b.flag, b.flagpos, b.ubQ, b.rowsQ);
     KMX_COUNT_LAUNCH();
-    tc_plan_back<<<kmx_stride_blocks(tq, 1, ctx->sm_count, 5), kTM, 0, st>>>(planQ, b.rowsQ, b.flagpos + nq_cap,
-                                                                            b.nitems + 3);
+    tc_lists<true><<<kListCtas * sms, kTM, 0, st>>>(planQ, b.rowsQ, b.flagpos + nq_cap, (int)grid, b.nitems + 4);
     KMX_COUNT_LAUNCH();
     tc_collect<true><<<grid, kThreads, smem, st>>>(dq, permQ, nq_cap, b.flagpos + nq_cap, b.rowsQ, b.packP, b.needQ, tp,
                                                    b.itemsQ, b.nitems + 1, b.ubQ, b.candQ, b.cntQ, ctx->d_err);
