@@ -18,10 +18,10 @@
 //             node's rows are split at a whole number of 128-row tiles
 //             (left: ceil(len / 256) * 128 rows) by their projection on the
 //             node's principal direction (power iteration on up to 256
-//             sampled rows).  The upper levels run level by level with one
-//             stable radix sort per level keyed by (side, node, quantised
-//             projection); below nodes of 16 tiles one CTA per node finishes
-//             its subtree in shared memory (bitonic sorts).  The leaves are
+//             sampled rows).  Level by level: nodes above 2048 rows by three
+//             launches (directions, keys of all rows, one CTA or cluster per
+//             node that splits by histograms and a stable partition), smaller
+//             ones by one (a CTA per node).  The leaves are
 //             the 128-row tiles, and they are tight: the rows of a tile are
 //             similar descriptors.
 //   pack      one CTA per 128-row tile: the tile centre, then per row
@@ -91,6 +91,7 @@
 #include "bulk_copy.cuh"
 #include "match_common.cuh"
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <float.h>
 
@@ -248,19 +249,15 @@ __device__ __forceinline__ void store_operand_row(uint8_t* tile, int r, const fl
 constexpr int kTreeSample = 256;  // rows sampled per node for its direction
 constexpr int kTreeIters = 2;     // power iterations
 constexpr int kTreeThreads = 256;
+constexpr int kTreeGrid = 1024;   // CTAs of tree_dir per side, at most
 constexpr int kDirStride = 68;    // floats per node: centre (33), direction (33), projection range (2)
-constexpr size_t kTreeSmem = sizeof(float) * kTreeSample * KMX_DESC_DIM;
-// Rows of a node tree_local splits in one CTA.  Its gathers of the node's
-// descriptor rows run on one SM, so a larger node is faster on the global
-// kernels, which spread a level over the whole GPU (on the 2M-point indoor
-// pair, 16384 beat 8192, 4096 and 65536).
-constexpr int kLocalRows = 16384;
-constexpr int kFinishLevels = 4;                         // levels below a node of 16 tiles
-constexpr int kFinishRows = kTM << kFinishLevels;        // 2048
-constexpr int kFinishSample = 256;                       // rows sampled per node below level0 (at most 2048 rows)
-// sampled rows, entries, partition buffer, 16-bit keys
-constexpr size_t kFinishSmem = sizeof(float) * kFinishSample * KMX_DESC_DIM + sizeof(int32_t) * 2 * kFinishRows +
-                               sizeof(uint16_t) * kFinishRows;
+// Rows of a node that one CTA splits from its descriptors to its two halves.
+// The CTA gathers the node's rows on one SM, so larger nodes get their keys
+// from a kernel over all rows (tree_key) and only then one CTA each
+// (tree_part).
+constexpr int kLocalRows = 2048;
+// the sampled rows, then the 16-bit keys of a node that is split at once
+constexpr size_t kTreeSmem = sizeof(float) * kTreeSample * KMX_DESC_DIM + sizeof(uint16_t) * kLocalRows;
 
 // Rows of the left child of a node of `len` rows: a whole number of tiles,
 // ceil(len / 256) * 128; a node of at most 128 rows is a leaf (its left
@@ -323,28 +320,20 @@ __host__ __device__ __forceinline__ int64_t level_max(int64_t n, int l)
     return n;
 }
 
-// The tree works on both clouds' rows packed together: entry e < np is
-// source row e, entry np + i target row i (np, nq the device counts).  They
-// start as the identity, and *n2 = np + nq.
-__global__ void __launch_bounds__(256) tree_init(int64_t np_cap, const int64_t* d_np, int64_t nq_cap,
-                                                 const int64_t* d_nq, int32_t* __restrict__ vals,
-                                                 int64_t* __restrict__ n2)
-{
-    const int64_t np = kmx_count(d_np, np_cap), nq = kmx_count(d_nq, nq_cap);
-    if (blockIdx.x == 0 && threadIdx.x == 0) *n2 = np + nq;
-    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < np + nq; e += (int64_t)gridDim.x * 256)
-        vals[e] = (int32_t)(e < np ? e : e - np);
-}
+// Both clouds' rows lie in one array: source row positions at [0, np), target
+// row positions at [tree_offset(np_cap), + nq) (np, nq the device counts), so
+// that a node's rows (its start is a multiple of 128) are 16-byte aligned.
+__host__ __device__ __forceinline__ int64_t tree_offset(int64_t np_cap) { return (np_cap + 7) / 8 * 8; }
 
-// The sorted rows into the layout the later stages read: source rows at
-// [0, np), target rows at [np_cap, np_cap + nq).
-__global__ void __launch_bounds__(256) tree_out(int64_t np_cap, const int64_t* d_np, int64_t nq_cap,
-                                                const int64_t* d_nq, const int32_t* __restrict__ vals,
-                                                int32_t* __restrict__ perm)
+// The rows start in their own order.
+__global__ void __launch_bounds__(256) tree_init(int64_t np_cap, const int64_t* d_np, int64_t nq_cap,
+                                                 const int64_t* d_nq, int32_t* __restrict__ vals)
 {
-    const int64_t np = kmx_count(d_np, np_cap), nq = kmx_count(d_nq, nq_cap);
-    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < np + nq; e += (int64_t)gridDim.x * 256)
-        perm[e < np ? e : np_cap + (e - np)] = vals[e];
+    const int64_t np = kmx_count(d_np, np_cap), nq = kmx_count(d_nq, nq_cap), off = tree_offset(np_cap);
+    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < np + nq; e += (int64_t)gridDim.x * 256) {
+        const int64_t i = e < np ? e : e - np;
+        vals[e < np ? i : off + i] = (int32_t)i;
+    }
 }
 
 // (x - c) . v over the 33 values of descriptor row x (16-byte aligned, read
@@ -540,59 +529,6 @@ __device__ void node_direction(const float* __restrict__ X, const int32_t* perm,
         }
 }
 
-// One CTA per (node of this level, side): the node's centre and principal
-// direction and the range of its sample's projections.  Leaves do nothing.
-__global__ void __launch_bounds__(kTreeThreads) tree_dir(const float* __restrict__ P, int64_t np_cap,
-                                                         const int64_t* d_np, const float* __restrict__ Q,
-                                                         int64_t nq_cap, const int64_t* d_nq,
-                                                         const int32_t* __restrict__ vals, int level,
-                                                         float* __restrict__ dirs)
-{
-    extern __shared__ float tree_smem[];
-    float(*xs)[KMX_DESC_DIM] = reinterpret_cast<float(*)[KMX_DESC_DIM]>(tree_smem);
-    __shared__ DirSmem<kTreeThreads> D;
-    const int side = blockIdx.y;
-    const int64_t k = blockIdx.x;
-    const int64_t np = kmx_count(d_np, np_cap), nq = kmx_count(d_nq, nq_cap);
-    if (level_max(np > nq ? np : nq, level) <= kLocalRows) return;  // tree_local takes this level
-    const int64_t n = side ? nq : np;
-    int64_t start, len;
-    tree_node(n, level, k, start, len);
-    if (len <= kTM) return;
-    float lo, hi;
-    node_direction(side ? Q : P, vals + (side ? kmx_count(d_np, np_cap) : 0) + start, len, xs, D, lo, hi);
-    float* d = dirs + (((int64_t)side << level) + k) * kDirStride;
-    const int tid = threadIdx.x;
-    if (tid < KMX_DESC_DIM) {
-        d[tid] = D.cvec[tid];
-        d[KMX_DESC_DIM + tid] = D.vvec[tid];
-    }
-    if (tid == 0) {
-        d[2 * KMX_DESC_DIM] = lo;
-        d[2 * KMX_DESC_DIM + 1] = hi;
-    }
-}
-
-// One tree level for nodes that fit in shared memory (at most kLocalRows
-// rows), one CTA of NT threads per (node, side), in one launch instead of
-// the direction, key and radix-sort launches of a global level.  The split
-// is the global levels' split: the first tree_left(len) rows in the order of
-// (16-bit key, position), the key being the projection on the node's
-// direction quantised over the sample's range.  That set is found without a
-// sort: two 256-bin histograms give the key T of the split row and how many
-// rows with key T go left; then a stable partition writes the left rows,
-// then the right rows, each in their current order, from src to dst.  Leaves
-// are copied.  A level that the global kernels ordered (some node of the
-// level larger than kLocalRows on the device) is left alone: their radix
-// sort wrote dst.
-constexpr size_t kLocalSmemBase = kTreeSmem;  // the sampled rows; the 16-bit keys follow
-constexpr int kLocalWideCtas = 304;           // from this many CTAs per level, CTAs of 256 threads (4 per SM)
-
-size_t local_smem_bytes(int64_t max_rows)
-{
-    return kLocalSmemBase + sizeof(uint16_t) * (size_t)((max_rows + 7) / 8 * 8);
-}
-
 // Smallest bin b with before + (hist[0] + ... + hist[b]) >= target, and the
 // count before it (bins in order), by warp 0 of the CTA; the result in
 // *bin / *below.
@@ -722,172 +658,296 @@ __device__ void split_at(const uint16_t* key, int len, int h, int* hist, int* se
     }
 }
 
-template <int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) tree_local(const float* __restrict__ P, int64_t np_cap,
-                                                           const int64_t* d_np, const float* __restrict__ Q,
-                                                           int64_t nq_cap, const int64_t* d_nq,
-                                                           const int32_t* __restrict__ src,
-                                                           int32_t* __restrict__ dst, int level, unsigned int* err)
+// One tree level, one CTA per (node of this level, side): the node's centre and
+// principal direction and the range of its sample's projections.  In a level
+// whose nodes hold at most kLocalRows rows (at the device counts) the CTA also
+// splits the node: the first tree_left(len) rows in the order of (16-bit key,
+// position), the key being the projection on the direction quantised over the
+// sample's range, go left, the others right, each in their current order, from
+// src to dst; leaves are copied.  In other levels it stores the direction for
+// tree_key and tree_part, which make the same split.  A split is a chain of
+// some twenty barriers (11 us for 2048 rows), so a level gets a CTA per node:
+// a CTA for all levels below 2048 rows, one node after another, took 300 us at
+// 302548 and 287858 rows, its four levels now take 240 us
+// (93 instead of 167 us at 40009 and 61003 rows).
+__global__ void __launch_bounds__(kTreeThreads, 4) tree_dir(const float* __restrict__ P, int64_t np_cap,
+                                                            const int64_t* d_np, const float* __restrict__ Q,
+                                                            int64_t nq_cap, const int64_t* d_nq,
+                                                            const int32_t* __restrict__ src,
+                                                            int32_t* __restrict__ dst, int level,
+                                                            float* __restrict__ dirs, unsigned int* err)
 {
-    constexpr int kWarpsL = NT / 32;
     extern __shared__ float tree_smem[];
     float(*xs)[KMX_DESC_DIM] = reinterpret_cast<float(*)[KMX_DESC_DIM]>(tree_smem);
     uint16_t* key = reinterpret_cast<uint16_t*>(tree_smem + kTreeSample * KMX_DESC_DIM);
-    __shared__ DirSmem<NT> D;
-    __shared__ int hist[256];
-    __shared__ int wsum[kWarpsL];
-    __shared__ int sel[4];   // B1, below B1, T, rows of key T that go left
-    __shared__ float range[2];
-    const int side = blockIdx.y;
-    const int tid = threadIdx.x;
-    const int64_t np = kmx_count(d_np, np_cap), nq = kmx_count(d_nq, nq_cap);
-    const int64_t n = side ? nq : np;
-    int64_t start, len64;
-    tree_node(n, level, blockIdx.x, start, len64);
-    const int32_t* gs = src + (side ? np : 0) + start;
-    int32_t* gd = dst + (side ? np : 0) + start;
-    // a level the global kernels ordered (their sort wrote dst) needs nothing
-    if (level_max(np > nq ? np : nq, level) > kLocalRows) return;
-    if (len64 <= kTM || len64 > kLocalRows) {  // a leaf (a larger node cannot occur): only the copy
-        if (len64 > kLocalRows && tid == 0) kmx_raise(err, KMX_DERR_CAPACITY);
-        for (int64_t i = tid; i < len64; i += NT) gd[i] = gs[i];
-        return;
-    }
-    const int len = (int)len64;
-    const int h = (int)tree_left(len64);  // 0 < h < len
-    const float* X = side ? Q : P;
-    float lo, hi;
-    node_direction(X, gs, len64, xs, D, lo, hi);
-    if (tid == 0) {
-        range[0] = lo;
-        range[1] = hi;
-    }
-    __syncthreads();
-    lo = range[0];
-    hi = range[1];
-    const float qs = hi > lo ? 65535.f / (hi - lo) : 0.f;
-    int32_t g = tid < len ? gs[tid] : 0;
-    for (int i = tid; i < len; i += NT) {
-        const int32_t gn = i + NT < len ? gs[i + NT] : 0;  // the next row's index, loaded during this row
-        const float p = project(X + (int64_t)g * KMX_DESC_STRIDE, D.cvec, D.vvec);
-        key[i] = (uint16_t)fminf(fmaxf((p - lo) * qs, 0.f), 65535.f);  // NaN -> 0
-        g = gn;
-    }
-    split_at<NT>(key, len, h, hist, sel, wsum, err, [&](int i) { return gs[i]; },
-                 [&](int pos, int32_t v) { gd[pos] = v; });
-}
-
-// The last levels of the tree, below `level0` (whose nodes hold at most
-// kFinishRows rows): one CTA per (level-0 node, side) splits its subtree
-// level by level in shared memory.  Per node: its direction (from up to
-// kFinishSample rows), 16-bit keys of all its rows and split_at, as
-// tree_local does; the next level splits each half again.  The entries are
-// read from src and written to vals (src may be vals).
-__global__ void __launch_bounds__(kTreeThreads) tree_finish(const float* __restrict__ P, int64_t np_cap,
-                                                            const int64_t* d_np, const float* __restrict__ Q,
-                                                            int64_t nq_cap, const int64_t* d_nq,
-                                                            const int32_t* src, int32_t* vals, int level0,
-                                                            int levels, unsigned int* err)
-{
-    extern __shared__ float tree_smem[];
-    float(*xs)[KMX_DESC_DIM] = reinterpret_cast<float(*)[KMX_DESC_DIM]>(tree_smem);
-    int32_t* perm = reinterpret_cast<int32_t*>(tree_smem + kFinishSample * KMX_DESC_DIM);  // [kFinishRows]
-    int32_t* tmp = perm + kFinishRows;                                                    // [kFinishRows]
-    uint16_t* key = reinterpret_cast<uint16_t*>(tmp + kFinishRows);                       // [kFinishRows]
-    __shared__ DirSmem<kTreeThreads, kFinishSample> D;
+    __shared__ DirSmem<kTreeThreads> D;
     __shared__ int hist[256];
     __shared__ int wsum[kTreeThreads / 32];
-    __shared__ int sel[4];
+    __shared__ int sel[4];  // B1, below B1, T, rows of key T that go left
     __shared__ float range[2];
     const int side = blockIdx.y;
     const int tid = threadIdx.x;
-    const int64_t np = kmx_count(d_np, np_cap);
-    const int64_t n = side ? kmx_count(d_nq, nq_cap) : np;
-    int64_t start, len;
-    tree_node(n, level0, blockIdx.x, start, len);
-    const float* X = side ? Q : P;
-    const int32_t* gs = src + (side ? np : 0) + start;
-    int32_t* gv = vals + (side ? np : 0) + start;
-    if (len <= kTM || len > kFinishRows) {  // a leaf (a larger node cannot occur): only the copy
-        if (len > kFinishRows && tid == 0) kmx_raise(err, KMX_DERR_CAPACITY);
-        if (gs != gv)
-            for (int64_t i = tid; i < len; i += kTreeThreads) gv[i] = gs[i];
+    const int64_t np = kmx_count(d_np, np_cap), nq = kmx_count(d_nq, nq_cap);
+    const int64_t n = side ? nq : np, off = side ? tree_offset(np_cap) : 0;
+    const int64_t largest = level_max(np > nq ? np : nq, level);
+    const bool local = largest <= kLocalRows;
+    if (largest <= kTM) {  // leaves only (levels that the capacities have and the counts do not)
+        for (int64_t i = (int64_t)blockIdx.x * kTreeThreads + tid; i < n; i += (int64_t)gridDim.x * kTreeThreads)
+            dst[off + i] = src[off + i];
         return;
     }
-    for (int i = tid; i < len; i += kTreeThreads) perm[i] = gs[i];
-    for (int l = level0; l < levels; ++l) {
-        const int sub = l - level0;
-        for (int c = 0; c < (1 << sub); ++c) {
-            // the sub-node's range within the CTA's rows
-            int64_t cs = 0, cl = len;
-            for (int b = sub - 1; b >= 0; --b) {
-                const int64_t h = tree_left(cl);
-                if ((c >> b) & 1) {
-                    cs += h;
-                    cl -= h;
-                } else {
-                    cl = h;
-                }
+    for (int64_t k = blockIdx.x; k < (int64_t{1} << level); k += gridDim.x) {
+        int64_t start, len64;
+        tree_node(n, level, k, start, len64);
+        const int32_t* gs = src + off + start;
+        int32_t* gd = dst + off + start;
+        if (len64 <= kTM) {  // a leaf
+            if (local)
+                for (int64_t i = tid; i < len64; i += kTreeThreads) gd[i] = gs[i];
+            continue;
+        }
+        const float* X = side ? Q : P;
+        float lo, hi;
+        node_direction(X, gs, len64, xs, D, lo, hi);
+        if (!local) {
+            float* d = dirs + (((int64_t)side << level) + k) * kDirStride;
+            if (tid < KMX_DESC_DIM) {
+                d[tid] = D.cvec[tid];
+                d[KMX_DESC_DIM + tid] = D.vvec[tid];
             }
-            if (cl <= kTM) continue;
-            float lo, hi;
-            node_direction(X, perm + cs, cl, xs, D, lo, hi);
             if (tid == 0) {
-                range[0] = lo;
-                range[1] = hi;
+                d[2 * KMX_DESC_DIM] = lo;
+                d[2 * KMX_DESC_DIM + 1] = hi;
             }
-            __syncthreads();
-            lo = range[0];
-            hi = range[1];
-            const float qs = hi > lo ? 65535.f / (hi - lo) : 0.f;
-            for (int i = tid; i < cl; i += kTreeThreads) {
-                const float p = project(X + (int64_t)perm[cs + i] * KMX_DESC_STRIDE, D.cvec, D.vvec);
+            continue;
+        }
+        if (tid == 0) {
+            range[0] = lo;
+            range[1] = hi;
+        }
+        __syncthreads();
+        lo = range[0];
+        hi = range[1];
+        const int len = (int)len64;
+        const float qs = hi > lo ? 65535.f / (hi - lo) : 0.f;
+        if (len <= kTreeSample) {  // the sample is the node: its centred rows are in shared memory
+            for (int i = tid; i < len; i += kTreeThreads) {
+                float p = 0.f;
+#pragma unroll
+                for (int h = 0; h < KMX_DESC_DIM; ++h) p = fmaf(xs[i][h], D.vvec[h], p);
                 key[i] = (uint16_t)fminf(fmaxf((p - lo) * qs, 0.f), 65535.f);  // NaN -> 0
             }
-            split_at<kTreeThreads>(key, (int)cl, (int)tree_left(cl), hist, sel, wsum, err,
-                                   [&](int i) { return perm[cs + i]; }, [&](int pos, int32_t v) { tmp[pos] = v; });
-            for (int i = tid; i < cl; i += kTreeThreads) perm[cs + i] = tmp[i];
-            // (the next node_direction starts with a barrier)
+        } else {
+            int32_t g = tid < len ? gs[tid] : 0;
+            for (int i = tid; i < len; i += kTreeThreads) {
+                const int32_t gn = i + kTreeThreads < len ? gs[i + kTreeThreads] : 0;  // loaded during this row
+                const float p = project(X + (int64_t)g * KMX_DESC_STRIDE, D.cvec, D.vvec);
+                key[i] = (uint16_t)fminf(fmaxf((p - lo) * qs, 0.f), 65535.f);
+                g = gn;
+            }
+        }
+        split_at<kTreeThreads>(key, len, (int)tree_left(len64), hist, sel, wsum, err, [&](int i) { return gs[i]; },
+                               [&](int pos, int32_t v) { gd[pos] = v; });
+    }
+}
+
+// The key of every row in a level of larger nodes: its projection on its node's
+// direction, quantised to 16 bits over the sample's range (leaves: none).
+__global__ void __launch_bounds__(256) tree_key(const float* __restrict__ P, int64_t np_cap, const int64_t* d_np,
+                                                const float* __restrict__ Q, int64_t nq_cap, const int64_t* d_nq,
+                                                const int32_t* __restrict__ vals, int level,
+                                                const float* __restrict__ dirs, uint16_t* __restrict__ keys)
+{
+    const int64_t np = kmx_count(d_np, np_cap), nq = kmx_count(d_nq, nq_cap), off = tree_offset(np_cap);
+    if (level_max(np > nq ? np : nq, level) <= kLocalRows) return;  // tree_dir split this level
+    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < np + nq; e += (int64_t)gridDim.x * 256) {
+        const int side = e >= np;
+        const int64_t pos = side ? e - np : e, at = side ? off + pos : pos;
+        int64_t start, len;
+        const int64_t k = tree_node_of(side ? nq : np, level, pos, start, len);
+        if (len <= kTM) continue;
+        const float* d = dirs + (((int64_t)side << level) + k) * kDirStride;
+        const float p = project((side ? Q : P) + (int64_t)vals[at] * KMX_DESC_STRIDE, d, d + KMX_DESC_DIM);
+        const float lo = d[2 * KMX_DESC_DIM], hi = d[2 * KMX_DESC_DIM + 1];
+        const float qs = hi > lo ? 65535.f / (hi - lo) : 0.f;
+        keys[at] = (uint16_t)fminf(fmaxf((p - lo) * qs, 0.f), 65535.f);
+    }
+}
+
+constexpr int kPartThreads = 1024;
+constexpr int kPartPer = 8;      // rows per lane and round
+constexpr int kPartCluster = 8;  // CTAs per node at most
+constexpr int kPartRows = kPartThreads * kPartPer;
+
+// The CTA's histogram h[256] of bin(key) (-1: none) over its keys, with one
+// copy per lane (copies[bin][lane]: no two lanes of a warp meet).  Ends with a
+// barrier.
+template <typename Bin>
+__device__ __forceinline__ void part_hist(const uint16_t* __restrict__ key, int len, int (*copies)[32], int* h, Bin bin)
+{
+    const int tid = threadIdx.x, lane = tid & 31;
+    for (int i = tid; i < 256 * 32; i += kPartThreads) (&copies[0][0])[i] = 0;
+    __syncthreads();
+    for (int b = tid; b < len; b += kPartRows) {
+        int k[kPartPer];
+#pragma unroll
+        for (int e = 0; e < kPartPer; ++e) {
+            const int i = b + e * kPartThreads;
+            k[e] = i < len ? bin((int)__ldg(key + i)) : -1;
+        }
+#pragma unroll
+        for (int e = 0; e < kPartPer; ++e)
+            if (k[e] >= 0) atomicAdd(&copies[k[e]][lane], 1);
+    }
+    __syncthreads();
+    // four threads per bin, eight copies each
+    int s = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) s += copies[tid >> 2][(tid & 3) * 8 + e];
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    if ((tid & 3) == 0) h[tid >> 2] = s;
+    __syncthreads();
+}
+
+// One cluster per node of a level that tree_dir does not split: the split of
+// tree_dir from the stored keys.  Each CTA takes a run of the node's rows.  Two
+// 256-bin histograms, summed over the cluster, give the key T of the split row
+// and how many rows with key T go left; the histograms of the CTAs before it
+// say where a CTA's left rows start, and a stable partition writes both halves,
+// 8192 rows per round, a warp's 32 rows of a step to consecutive places.  What
+// bounds it: those rounds on one SM per CTA, so the few large nodes of the
+// first levels get up to eight CTAs.  302548 and 287858 rows: 30 us for
+// the first level, 13 to 23 us for the seven others; a radix sort of a level over
+// the whole GPU, six launches, took 62 us.
+__global__ void __launch_bounds__(kPartThreads) tree_part(int64_t np_cap, const int64_t* d_np, int64_t nq_cap,
+                                                          const int64_t* d_nq, const int32_t* __restrict__ src,
+                                                          int32_t* __restrict__ dst,
+                                                          const uint16_t* __restrict__ keys, int level,
+                                                          unsigned int* err)
+{
+    namespace cg = cooperative_groups;
+    __shared__ int copies[256][32];
+    __shared__ int h1[256], h2[256], sum[256];
+    __shared__ int sel[4];
+    __shared__ int before[2];
+    __shared__ int2 wsum[2][32];  // per round (two in turn) and warp: rows with key < T and with key T
+    const int64_t np = kmx_count(d_np, np_cap), nq = kmx_count(d_nq, nq_cap);
+    if (level_max(np > nq ? np : nq, level) <= kLocalRows) return;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int ctas = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int side = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int64_t start, len64;
+    tree_node(side ? nq : np, level, blockIdx.x / ctas, start, len64);
+    const int64_t at = (side ? tree_offset(np_cap) : 0) + start;
+    int32_t* gd = dst + at;
+    if (len64 <= kTM) {  // the whole cluster
+        if (rank == 0)
+            for (int64_t i = tid; i < len64; i += kPartThreads) gd[i] = src[at + i];
+        return;
+    }
+    const int node = (int)len64, h = (int)tree_left(len64);
+    const int run = (node + ctas - 1) / ctas, first = min(rank * run, node), len = min(run, node - first);
+    const uint16_t* key = keys + at + first;
+    const int32_t* gs = src + at + first;
+    part_hist(key, len, copies, h1, [](int k) { return k >> 8; });
+    cluster.sync();
+    if (tid < 256) {
+        int s = 0;
+        for (int c = 0; c < ctas; ++c) s += cluster.map_shared_rank(h1, c)[tid];
+        sum[tid] = s;
+    }
+    __syncthreads();
+    if (warp == 0) select_bin(sum, 0, h, &sel[0], &sel[1]);
+    __syncthreads();
+    const int b1 = sel[0], below1 = sel[1];
+    part_hist(key, len, copies, h2, [b1](int k) { return (k >> 8) == b1 ? k & 0xff : -1; });
+    cluster.sync();
+    if (tid < 256) {
+        int s = 0;
+        for (int c = 0; c < ctas; ++c) s += cluster.map_shared_rank(h2, c)[tid];
+        sum[tid] = s;
+    }
+    if (tid < 2) before[tid] = 0;
+    __syncthreads();
+    if (warp == 0) {
+        int b2, below2;
+        select_bin(sum, below1, h, &b2, &below2);
+        if (lane == 0) {
+            sel[2] = (b1 << 8) | b2;
+            sel[3] = h - below2;
         }
     }
     __syncthreads();
-    for (int i = tid; i < len; i += kTreeThreads) gv[i] = perm[i];
-}
-
-// Sort key of every packed entry for this level: side (top bit), node index
-// (level bits), then the row's projection on its node's direction,
-// quantised over the sample's range (0 in a leaf).  *n_sort gets the count
-// the radix sort takes (0 when tree_local takes the level).
-__global__ void __launch_bounds__(256) tree_key(const float* __restrict__ P, int64_t np_cap, const int64_t* d_np,
-                                                const float* __restrict__ Q, int64_t nq_cap, const int64_t* d_nq,
-                                                const int32_t* __restrict__ vals, int level, int key_bits,
-                                                const float* __restrict__ dirs, uint32_t* __restrict__ keys,
-                                                int64_t* __restrict__ n_sort)
-{
-    const int64_t np = kmx_count(d_np, np_cap), nq = kmx_count(d_nq, nq_cap);
-    // the entries this level's radix sort orders: all of them, or none when
-    // every node fits tree_local
-    const bool global = level_max(np > nq ? np : nq, level) > kLocalRows;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *n_sort = global ? np + nq : 0;
-    if (!global) return;
-    const int pbits = key_bits - 1 - level;
-    const int qbits = pbits < 22 ? pbits : 22;
-    const float qmax = (float)((1u << qbits) - 1u);
-    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < np + nq; e += (int64_t)gridDim.x * 256) {
-        const int side = e >= np;
-        const int64_t pos = side ? e - np : e;
-        int64_t start, len;
-        const int64_t k = tree_node_of(side ? nq : np, level, pos, start, len);
-        uint32_t q = 0;
-        if (len > kTM) {
-            const float* d = dirs + (((int64_t)side << level) + k) * kDirStride;
-            const float* x = (side ? Q : P) + (int64_t)vals[e] * KMX_DESC_STRIDE;
-            const float p = project(x, d, d + KMX_DESC_DIM);
-            const float lo = d[2 * KMX_DESC_DIM], hi = d[2 * KMX_DESC_DIM + 1];
-            const float t = hi > lo ? (p - lo) / (hi - lo) * qmax : 0.f;
-            q = (uint32_t)fminf(fmaxf(t, 0.f), qmax) << (pbits - qbits);
+    const int T = sel[2], need = sel[3];
+    if (tid < 256) {  // rows with key < T and with key T in the CTAs before this one
+        const int b2 = T & 0xff;
+        int l = 0, e = 0;
+        for (int c = 0; c < rank; ++c) {
+            if (tid < b1) l += cluster.map_shared_rank(h1, c)[tid];
+            const int x = cluster.map_shared_rank(h2, c)[tid];
+            if (tid < b2) l += x;
+            if (tid == b2) e += x;
         }
-        keys[e] = ((uint32_t)side << (key_bits - 1)) | ((uint32_t)k << pbits) | q;
+        l = __reduce_add_sync(0xffffffffu, l);
+        e = __reduce_add_sync(0xffffffffu, e);
+        if (lane == 0) {
+            atomicAdd(&before[0], l);
+            atomicAdd(&before[1], e);
+        }
+    }
+    cluster.sync();  // the others' histograms are read
+    int run_l = before[0], run_e = before[1];  // key < T, key == T so far (uniform)
+    // the warp's rows of a round: 256 consecutive ones, 32 to a step
+    const int mine0 = warp * 32 * kPartPer + lane;
+    int k[kPartPer];
+    int32_t v[kPartPer];
+    auto fetch = [&](int b) {
+#pragma unroll
+        for (int e = 0; e < kPartPer; ++e) {
+            const int i = b + mine0 + 32 * e;
+            k[e] = i < len ? (int)__ldg(key + i) : 0x10000;
+            v[e] = i < len ? __ldg(gs + i) : 0;
+        }
+    };
+    fetch(0);
+    const unsigned lt = (1u << lane) - 1u;
+    int phase = 0;
+    for (int b = 0; b < len; b += kPartRows, phase ^= 1) {
+        int kc[kPartPer];
+        int32_t vc[kPartPer];
+        int wl = 0, we = 0;
+#pragma unroll
+        for (int e = 0; e < kPartPer; ++e) {
+            kc[e] = k[e];
+            vc[e] = v[e];
+            wl += __popc(__ballot_sync(0xffffffffu, kc[e] < T));
+            we += __popc(__ballot_sync(0xffffffffu, kc[e] == T));
+        }
+        fetch(b + kPartRows);  // the next round's, during this one
+        if (lane == 0) wsum[phase][warp] = make_int2(wl, we);
+        __syncthreads();
+        const int2 t = wsum[phase][lane];
+        int nl = run_l + __reduce_add_sync(0xffffffffu, lane < warp ? t.x : 0);
+        int ne = run_e + __reduce_add_sync(0xffffffffu, lane < warp ? t.y : 0);
+        run_l += __reduce_add_sync(0xffffffffu, t.x);
+        run_e += __reduce_add_sync(0xffffffffu, t.y);
+#pragma unroll
+        for (int e = 0; e < kPartPer; ++e) {
+            const int i = b + mine0 + 32 * e;
+            const unsigned bl = __ballot_sync(0xffffffffu, kc[e] < T), be = __ballot_sync(0xffffffffu, kc[e] == T);
+            const int l = nl + __popc(bl & lt), q = ne + __popc(be & lt);  // of the node's rows before this one
+            nl += __popc(bl);
+            ne += __popc(be);
+            if (i >= len) continue;
+            const int left_before = l + min(q, need);
+            const bool left = kc[e] < T || (kc[e] == T && q < need);
+            const int to = left ? left_before : h + (first + i - left_before);
+            if (to < node)  // always (the counts add up to h left rows); checked, not assumed
+                gd[to] = vc[e];
+            else
+                kmx_raise(err, KMX_DERR_CAPACITY);
+        }
     }
 }
 
@@ -2014,19 +2074,32 @@ __global__ void __launch_bounds__(256) fallback_merge(const kmx::RowBest* __rest
     }
 }
 
+cudaError_t tree_part_launch(cudaStream_t st, int ctas, int level, int64_t np_cap, const int64_t* d_np, int64_t nq_cap,
+                             const int64_t* d_nq, const int32_t* src, int32_t* dst, const uint16_t* keys,
+                             unsigned int* err)
+{
+    cudaLaunchAttribute cluster{};
+    cluster.id = cudaLaunchAttributeClusterDimension;
+    cluster.val.clusterDim.x = (unsigned)ctas;
+    cluster.val.clusterDim.y = 1;
+    cluster.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)ctas << level, 2);
+    cfg.blockDim = dim3(kPartThreads);
+    cfg.stream = st;
+    cfg.attrs = &cluster;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, tree_part, np_cap, d_np, nq_cap, d_nq, src, dst, keys, level, err);
+}
+
 size_t tc_smem_bytes()
 {
     return sizeof(TcShared) + 1024;
 }
 
 struct TcBuffers {
-    uint32_t *keys, *keys_tmp;
-    int32_t *vals, *vals_tmp;  // the tree's packed entries (source rows, then target rows), level to level
-    int32_t* vals_sort;        // the radix sort's temporary values
-    int32_t* perm;             // sorted: [0, np) source rows, [np_cap, np_cap + nq) target rows
-    int64_t* n2;               // np + nq on the device
-    int64_t* nsort;            // the entries a global level's radix sort takes (np + nq or 0)
-    void* sort_scratch;
+    uint16_t* keys;            // the tree's projections of a level
+    int32_t* vals[2];          // the rows in the order of a level: a level reads one and writes the other (tree_offset)
     float* dirs;               // [2 << (levels - 1)][kDirStride]
     uint8_t *packP, *packQ;
     float *cenP, *cenQ;
@@ -2058,15 +2131,12 @@ TcBuffers tc_carve(void* base, int64_t np_cap, int64_t nq_cap, size_t* total)
     const int64_t tp = (np_cap + kTN - 1) / kTN, tq = (nq_cap + kTN - 1) / kTN;  // tiles of either cloud
     const int levels = tc_levels(np_cap, nq_cap);
     const int fc = kmx_match_fp32_max_chunks();
-    b.keys = (uint32_t*)a.take(sizeof(uint32_t) * (size_t)n2);
-    b.keys_tmp = (uint32_t*)a.take(sizeof(uint32_t) * (size_t)n2);
-    b.vals = (int32_t*)a.take(sizeof(int32_t) * (size_t)n2);
-    b.vals_tmp = (int32_t*)a.take(sizeof(int32_t) * (size_t)n2);
-    b.vals_sort = (int32_t*)a.take(sizeof(int32_t) * (size_t)n2);
-    b.perm = (int32_t*)a.take(sizeof(int32_t) * (size_t)n2);
-    b.n2 = (int64_t*)a.take(sizeof(int64_t));
-    b.nsort = (int64_t*)a.take(sizeof(int64_t));
-    b.sort_scratch = a.take(kmx_sort_scratch_bytes(n2));
+    const int64_t nt = tree_offset(np_cap) + nq_cap;
+    b.keys = (uint16_t*)a.take(sizeof(uint16_t) * (size_t)(nt + 8));
+    b.vals[0] = (int32_t*)a.take(sizeof(int32_t) * (size_t)(nt + 8));
+    b.vals[1] = (int32_t*)a.take(sizeof(int32_t) * (size_t)(nt + 8));
+    b.flag = (int32_t*)a.take(sizeof(int32_t) * (size_t)(nq_cap + 1));
+    b.rowsQ = (int32_t*)a.take(sizeof(int32_t) * (size_t)nq_cap);
     b.dirs = (float*)a.take(sizeof(float) * kDirStride * ((size_t)2 << (levels > 0 ? levels - 1 : 0)));
     b.packP = (uint8_t*)a.take((size_t)tp * kColBytes);
     b.packQ = (uint8_t*)a.take((size_t)tq * kColBytes);
@@ -2091,8 +2161,6 @@ TcBuffers tc_carve(void* base, int64_t np_cap, int64_t nq_cap, size_t* total)
     b.nneedQ = b.nneedP + tp;
     b.cntP = b.nneedQ + tq;
     b.cntQ = b.cntP + np_cap;
-    b.flag = (int32_t*)b.keys;      // the tree's keys and entries are no longer needed then
-    b.rowsQ = b.vals_tmp;
     b.flagpos = (int64_t*)a.take(sizeof(int64_t) * (size_t)(nq_cap + 1));
     b.candP = (int32_t*)a.take(sizeof(int32_t) * kCandCap * (size_t)np_cap);
     b.candQ = (int32_t*)a.take(sizeof(int32_t) * kCandCap * (size_t)nq_cap);
@@ -2123,7 +2191,6 @@ cudaError_t kmx_match_tc_launch(kmx_ctx* ctx, const float* dp, int64_t np_cap, c
     const int64_t n2 = np_cap + nq_cap;
     const int64_t tp = (np_cap + kTN - 1) / kTN, tq = (nq_cap + kTN - 1) / kTN;
     const int levels = tc_levels(np_cap, nq_cap);
-    const int key_bits = levels <= 14 ? 24 : 32;
     if (levels > 30) return cudaErrorInvalidValue;
     const size_t smem = tc_smem_bytes();
     cudaError_t e = kmx_once_per_device(kmx_attr_tc_topk, [smem] {
@@ -2131,70 +2198,32 @@ cudaError_t kmx_match_tc_launch(kmx_ctx* ctx, const float* dp, int64_t np_cap, c
         if (r) return r;
         r = cudaFuncSetAttribute(tc_collect<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (r) return r;
-        r = cudaFuncSetAttribute(tree_dir, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTreeSmem);
-        if (r) return r;
-        r = cudaFuncSetAttribute(tree_local<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)local_smem_bytes(kLocalRows));
-        if (r) return r;
-        r = cudaFuncSetAttribute(tree_local<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)local_smem_bytes(kLocalRows));
-        if (r) return r;
-        return cudaFuncSetAttribute(tree_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFinishSmem);
+        return cudaFuncSetAttribute(tree_dir, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTreeSmem);
     });
     if (e) return e;
     if ((e = cudaMemsetAsync(b.nlist, 0, b.zeroed, st))) return e;
-    // locality order of both clouds: one tree level per sort
+    // locality order of both clouds, a tree level at a time
     const unsigned gb = kmx_stride_blocks(n2, 256, ctx->sm_count);
     KMX_COUNT_LAUNCH();
-    tree_init<<<gb, 256, 0, st>>>(np_cap, d_np, nq_cap, d_nq, b.vals, b.n2);
-    const int level0 = levels > kFinishLevels ? levels - kFinishLevels : 0;
-    // Levels whose nodes can exceed kLocalRows at the capacities run the
-    // global kernels (direction, keys, radix sort), which do nothing on the
-    // device once every node fits; tree_local then splits the level (or,
-    // after the global kernels, does nothing).  The entries alternate
-    // between vals and vals_tmp: the sort and tree_local read one and write
-    // the other.
+    tree_init<<<gb, 256, 0, st>>>(np_cap, d_np, nq_cap, d_nq, b.vals[0]);
     int64_t node_max = np_cap > nq_cap ? np_cap : nq_cap;  // largest node of level l at any device count
-    int32_t* cur = b.vals;                                  // the entries as the last level left them
-    for (int l = 0; l < level0; ++l, node_max = tree_left(node_max)) {
-        int32_t* next = cur == b.vals ? b.vals_tmp : b.vals;
-        if (node_max > kLocalRows) {
-            KMX_COUNT_LAUNCH();
-            tree_dir<<<dim3(1u << l, 2), kTreeThreads, kTreeSmem, st>>>(dp, np_cap, d_np, dq, nq_cap, d_nq, cur, l,
-                                                                         b.dirs);
-            KMX_COUNT_LAUNCH();
-            // 16-bit keys (two radix passes) while they leave at least 9 bits
-            // of projection (levels 0..6), wider keys below
-            const int kb = l <= 6 ? 16 : key_bits;
-            tree_key<<<gb, 256, 0, st>>>(dp, np_cap, d_np, dq, nq_cap, d_nq, cur, l, kb, b.dirs, b.keys, b.nsort);
-            if ((e = cudaGetLastError())) return e;
-            if ((e = kmx_sort_u32(ctx, b.keys, cur, b.keys_tmp, b.vals_sort, n2, b.nsort, kb, b.sort_scratch,
-                                  next)))
-                return e;
-        }
-        const int64_t rows = node_max < kLocalRows ? node_max : kLocalRows;
+    int cur = 0;                                            // the rows as the last level left them
+    for (int l = 0; l < levels; ++l, node_max = tree_left(node_max), cur ^= 1) {
         KMX_COUNT_LAUNCH();
-        if ((int64_t{2} << l) >= kLocalWideCtas) {
-            tree_local<256><<<dim3(1u << l, 2), 256, local_smem_bytes(rows), st>>>(dp, np_cap, d_np, dq, nq_cap,
-                                                                                  d_nq, cur, next, l, ctx->d_err);
-        } else {
-            tree_local<1024><<<dim3(1u << l, 2), 1024, local_smem_bytes(rows), st>>>(dp, np_cap, d_np, dq, nq_cap,
-                                                                                    d_nq, cur, next, l, ctx->d_err);
-        }
-        if ((e = cudaGetLastError())) return e;
-        cur = next;
-    }
-    if (levels > 0) {  // the subtrees of at most 16 tiles, one CTA each
+        tree_dir<<<dim3(l < 10 ? 1u << l : (unsigned)kTreeGrid, 2), kTreeThreads, kTreeSmem, st>>>(dp, np_cap, d_np, dq, nq_cap, d_nq, b.vals[cur],
+                                                                     b.vals[cur ^ 1], l, b.dirs, ctx->d_err);
+        if (node_max <= kLocalRows) continue;  // tree_dir splits the level at every device count
         KMX_COUNT_LAUNCH();
-        tree_finish<<<dim3(1u << level0, 2), kTreeThreads, kFinishSmem, st>>>(dp, np_cap, d_np, dq, nq_cap, d_nq,
-                                                                             cur, b.vals, level0, levels,
-                                                                             ctx->d_err);
-        if ((e = cudaGetLastError())) return e;
+        tree_key<<<gb, 256, 0, st>>>(dp, np_cap, d_np, dq, nq_cap, d_nq, b.vals[cur], l, b.dirs, b.keys);
+        KMX_COUNT_LAUNCH();
+        const int ctas = l < 3 ? kPartCluster : l == 3 ? 4 : l == 4 ? 2 : 1;  // at most 64 while clusters are used
+        if ((e = tree_part_launch(st, ctas, l, np_cap, d_np, nq_cap, d_nq, b.vals[cur], b.vals[cur ^ 1], b.keys,
+                                  ctx->d_err)))
+            return e;
     }
-    KMX_COUNT_LAUNCH();
-    tree_out<<<gb, 256, 0, st>>>(np_cap, d_np, nq_cap, d_nq, b.vals, b.perm);
-    const int32_t* permP = b.perm;
-    const int32_t* permQ = b.perm + np_cap;
+    if ((e = cudaGetLastError())) return e;
+    const int32_t* permP = b.vals[cur];
+    const int32_t* permQ = b.vals[cur] + tree_offset(np_cap);
     // packed tiles, centres and radii
     KMX_COUNT_LAUNCH();
     tc_pack<<<kmx_stride_blocks(tp, 1, ctx->sm_count, 16), kTN, 0, st>>>(dp, permP, np_cap, d_np, b.packP, b.cenP,
