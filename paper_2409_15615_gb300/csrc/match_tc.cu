@@ -128,6 +128,7 @@ constexpr int kCandCap = 512;                 // candidate list per row
 constexpr int kItemTiles = 32;                // column tiles per work item, at most
 constexpr int kItemMin = 8;                   // and at least, but for the last of a list
 constexpr int kItemsPerCta = 6;               // wanted, as far as kItemMin allows
+constexpr int kHeavyRow = 48;                 // candidates of a row from which tc_rerank gives it a whole warp
 constexpr int kListSeg = 32;                  // column tiles, the unit by which a row tile's list is cut among CTAs
 constexpr int kPlanRec = 32;                  // columns of the nearest tile recorded per row in the plan
 constexpr int kCandBuf = 16;                  // candidates buffered per row in the collect kernel
@@ -1960,7 +1961,10 @@ __device__ __forceinline__ void put_summary(int i, float d1, int j1, float d2, k
 }
 
 // Four sorted row positions per warp, eight lanes each (lane s takes
-// candidates s, s + 8, ...).  Rows whose list overflowed are appended to the
+// candidates s, s + 8, ...); a row with more than kHeavyRow candidates takes the
+// whole warp, because a lane's candidates are a chain of gathers and the
+// longest row ends the kernel: 40009 x
+// 61003 rows, 8 candidates a row: 86 -> 47 us.  Rows whose list overflowed are appended to the
 // exact fallback's list (in any order: each row's summary is its own).
 __global__ void __launch_bounds__(256) tc_rerank(const float* __restrict__ X, const int32_t* __restrict__ permX,
                                                  int64_t nx_cap, const int64_t* d_nx, const float* __restrict__ Y,
@@ -1984,30 +1988,23 @@ __global__ void __launch_bounds__(256) tc_rerank(const float* __restrict__ X, co
         const int orig = active ? permX[i] : 0;
         // target rows that are no source row's nearest stay out
         const int c = active && (rows_out || colbest[orig] != ~0ull) ? cnt[i] : 0;
+        const bool heavy = c > kHeavyRow && c <= kCandCap;
         float b1 = INFINITY, b2 = INFINITY;
         int j1 = 0x7fffffff;
-        if (c <= kCandCap && c > s) {
+        // candidates q0, q0 + step, ... of the c of row i
+        auto take = [&](int64_t i, int orig, int c, int q0, int step) {
             // the row once, then every candidate with the exact path's arithmetic
             // (one fused multiply-add per term in h order)
             float x[KMX_DESC_DIM];
-            const float4* x4 = reinterpret_cast<const float4*>(X + (int64_t)orig * KMX_DESC_STRIDE);
-    #pragma unroll
-            for (int q4 = 0; q4 < 8; ++q4) {
-                const float4 v = __ldg(x4 + q4);
-                x[4 * q4] = v.x;
-                x[4 * q4 + 1] = v.y;
-                x[4 * q4 + 2] = v.z;
-                x[4 * q4 + 3] = v.w;
-            }
-            x[32] = __ldg(X + (int64_t)orig * KMX_DESC_STRIDE + 32);
-            for (int q = s; q < c; q += 8) {
+            load_row(X + (int64_t)orig * KMX_DESC_STRIDE, true, x);
+            for (int q = q0; q < c; q += step) {
                 const int pos = cand[i * kCandCap + q];
                 if (pos < 0 || pos >= ny) continue;  // padding columns are never collected
                 const int j = permY[pos];
                 const float* y = Y + (int64_t)j * KMX_DESC_STRIDE;
                 const float4* y4 = reinterpret_cast<const float4*>(y);
                 float acc = 0.f;
-    #pragma unroll
+#pragma unroll
                 for (int q4 = 0; q4 < 8; ++q4) {
                     const float4 v = __ldg(y4 + q4);
                     float e = x[4 * q4] - v.x;
@@ -2023,20 +2020,36 @@ __global__ void __launch_bounds__(256) tc_rerank(const float* __restrict__ X, co
                 acc = fmaf(e, e, acc);
                 kmx::row_update(b1, j1, b2, acc, j);
             }
-        }
-    #pragma unroll
-        for (int o = 4; o >= 1; o >>= 1) {  // within the row's eight lanes
+        };
+        auto merge = [&](int o) {
             const float od1 = __shfl_xor_sync(0xffffffffu, b1, o);
             const int oj = __shfl_xor_sync(0xffffffffu, j1, o);
             const float od2 = __shfl_xor_sync(0xffffffffu, b2, o);
             kmx::row_merge(b1, j1, b2, od1, oj, od2);
+        };
+        if (!heavy && c <= kCandCap && c > s) take(i, orig, c, s, 8);
+#pragma unroll
+        for (int o = 4; o >= 1; o >>= 1) merge(o);  // within the row's eight lanes
+        if (s == 0 && active && !heavy) {
+            if (c > kCandCap)
+                fb_list[atomicAdd(reinterpret_cast<unsigned long long*>(fb_n), 1ull)] = orig;  // at most nx entries
+            else
+                put_summary(orig, b1, j1, b2, rows_out, colbest);
         }
-        if (s != 0 || !active) continue;
-        if (c > kCandCap) {
-            fb_list[atomicAdd(reinterpret_cast<unsigned long long*>(fb_n), 1ull)] = orig;  // at most nx entries
-            continue;
+        // rows with many candidates, one after the other over the whole warp
+        unsigned todo = __ballot_sync(0xffffffffu, heavy && s == 0);
+        while (todo) {
+            const int from = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const int horig = __shfl_sync(0xffffffffu, orig, from), hc = __shfl_sync(0xffffffffu, c, from);
+            b1 = INFINITY;
+            b2 = INFINITY;
+            j1 = 0x7fffffff;
+            if (lane < hc) take(base + (from >> 3), horig, hc, lane, 32);
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) merge(o);
+            if (lane == 0) put_summary(horig, b1, j1, b2, rows_out, colbest);
         }
-        put_summary(orig, b1, j1, b2, rows_out, colbest);
     }
 }
 
