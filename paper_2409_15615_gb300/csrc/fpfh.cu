@@ -281,7 +281,7 @@ cudaError_t kmx_fasterpfh_launch(kmx_ctx* ctx, const kmx_grid* g, const kmx_para
     spfh_kernel<<<nbs, kThreads, 0, st>>>(n, g->d_n, g->pts, reinterpret_cast<const float4*>(normal4), flags,
                                           offs, nbr, nbr_cap, prm->tau_num, g->sorted, g->d_n_sorted, sp, s.jflag,
                                           s.wlist, s.wcnt);
-    if ((e = kmx_scan_i32(ctx, s.jflag, n, g->d_n, s.jpos))) return e;
+    if ((e = kmx_scan_i32_live(ctx, s.jflag, n, g->d_n, s.jpos))) return e;
     KMX_COUNT_LAUNCH();
     scatter_valid<<<kmx_stride_blocks(n, kThreads, ctx->sm_count), kThreads, 0, st>>>(n, g->d_n, s.jflag, s.jpos,
                                                                                        valid, n_valid);

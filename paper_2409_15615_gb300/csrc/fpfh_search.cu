@@ -426,7 +426,7 @@ cudaError_t kmx_fpfh_search_launch(kmx_ctx* ctx, const kmx_grid* g, const kmx_pa
         KMX_COUNT_LAUNCH();
         valid_walk<<<nbw, kThreads, 0, st>>>(gv, R, prm->tau_num, flags, s.jflag);
     }
-    if ((e = kmx_scan_i32(ctx, s.jflag, n, g->d_n, s.jpos))) return e;
+    if ((e = kmx_scan_i32_live(ctx, s.jflag, n, g->d_n, s.jpos))) return e;
     KMX_COUNT_LAUNCH();
     scatter_j<<<kmx_stride_blocks(n, kThreads, ctx->sm_count), kThreads, 0, st>>>(n, g->d_n, s.jflag, s.jpos, valid,
                                                                                    n_valid);

@@ -102,7 +102,7 @@ cudaError_t match_emit(kmx_ctx* ctx, const MatchScratch& s, int64_t np_cap, cons
 {
     cudaStream_t st = ctx->stream;
     cudaError_t e;
-    if ((e = kmx_scan_i32(ctx, s.mflag, np_cap, d_np, s.mpos))) return e;
+    if ((e = kmx_scan_i32_live(ctx, s.mflag, np_cap, d_np, s.mpos))) return e;
     KMX_COUNT_LAUNCH();
     emit<<<kmx_stride_blocks(np_cap, kThreads, ctx->sm_count), kThreads, 0, st>>>(np_cap, d_np, s.merged, s.mflag,
                                                                                    s.mpos, vp, vq, out, cap, n_out,

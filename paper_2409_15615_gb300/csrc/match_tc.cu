@@ -2278,7 +2278,7 @@ cudaError_t kmx_match_tc_launch(kmx_ctx* ctx, const float* dp, int64_t np_cap, c
     KMX_COUNT_LAUNCH();
     back_flag<<<qb, 256, 0, st>>>(permQ, nq_cap, d_nq, s.colbest, b.flag);
     if ((e = cudaGetLastError())) return e;
-    if ((e = kmx_scan_i32(ctx, b.flag, nq_cap, d_nq, b.flagpos))) return e;
+    if ((e = kmx_scan_i32_live(ctx, b.flag, nq_cap, d_nq, b.flagpos))) return e;
     KMX_COUNT_LAUNCH();
     back_rows<<<qb, 256, 0, st>>>(permQ, nq_cap, d_nq, s.colbest, b.flag, b.flagpos, b.ubQ, b.rowsQ);
     KMX_COUNT_LAUNCH();
