@@ -69,7 +69,14 @@ constexpr int kCtasPerSm = 2;
 constexpr int kChunksPerCta = 8;      // default chunks of the tile sequence per resident CTA (load balance)
 constexpr int kMaxChunksPerCta = 32;  // the largest setting (kmx_set_match_chunks)
 constexpr int kTailChunksPerCta = 4;  // smaller chunks per CTA for the end of the sequence
-constexpr int kMinChunk = 4;       // tile pairs per chunk at least (more than kStages - 1)
+constexpr int kMinChunk = 4;       // tile pairs per chunk at least (more than kStages - 1), but for small matches
+// Small matches (below kSmallPairs tile pairs per CTA at the capacities) take
+// chunks down to one tile pair, so that every CTA gets work: 1021 x 897 rows are
+// 64 tile pairs, 38 us in 16 chunks of 4, 20 us in 64.  The ids of the chunks
+// in the ring are then more than two; the kernel for other matches keeps two.
+constexpr int kSmallPairs = 8;
+constexpr int kChunkIds = 8;
+static_assert(kChunkIds > kStages + 1, "the items in the ring and the current one may all be of different chunks");
 
 // Thread 0's position in its own stream of tile pairs (kept in shared memory:
 // only thread 0 uses it): the chunk being produced, the offset in it, the tile
@@ -109,7 +116,7 @@ struct __align__(16) BulkShared {
     uint64_t bar_q[kStages];
     Producer prod;
     ChunkGeo cg;                                        // the chunk geometry (thread 0 writes it once)
-    int chunk[2];                                       // chunk ids of the current and next local chunk
+    int chunk[kChunkIds];                               // ids of the current and next local chunks, in turn
     int end_item;                                       // first local item past the stream (INT_MAX = unknown)
     int failed;
 };
@@ -314,17 +321,18 @@ __device__ __forceinline__ void row_step(unsigned long long& k1, float& b2, floa
 
 constexpr unsigned long long kNoBest = (0x7f800000ull << 32) | 0x7fffffffull;  // (+inf, no column)
 
-__device__ __forceinline__ ChunkGeo chunk_geo(int64_t W, int ctas, int chunks_per_cta)
+__device__ __forceinline__ ChunkGeo chunk_geo(int64_t W, int ctas, int chunks_per_cta, bool small)
 {
     const int64_t per = (int64_t)chunks_per_cta * ctas;
     int64_t LA = (W + per - 1) / per;
-    if (LA < kMinChunk) LA = kMinChunk;
+    const int64_t least = small ? min((int64_t)kMinChunk, max((int64_t)1, W / (2 * (int64_t)ctas))) : kMinChunk;
+    if (LA < least) LA = least;
     const int64_t tail = W < ctas * LA ? W : ctas * LA;
     const int64_t NA = (W - tail) / LA;
     const int64_t WA = NA * LA;
     const int64_t tper = (int64_t)kTailChunksPerCta * ctas;
     int64_t LB = (W - WA + tper - 1) / tper;
-    if (LB < kMinChunk) LB = kMinChunk;
+    if (LB < least) LB = least;
     const int64_t NB = (W - WA + LB - 1) / LB;
     return ChunkGeo{(int)LA, (int)NA, (int)LB, (int)(NA + NB), WA};
 }
@@ -347,6 +355,7 @@ __device__ __forceinline__ int read_end(const BulkShared& S) { return *reinterpr
 // current one is used up, stop (recording the end of the stream) when the
 // counter has run out or the tile sequence has ended, else issue the copies
 // of the item's column tile into its ring stage.
+template <int kIds>
 __device__ __forceinline__ bool produce(BulkShared& S, int u, const ChunkGeo& cg, int64_t W, int nqt,
                                         int32_t* counter, const float* __restrict__ qn,
                                         const int32_t* __restrict__ qperm,
@@ -354,7 +363,7 @@ __device__ __forceinline__ bool produce(BulkShared& S, int u, const ChunkGeo& cg
 {
     Producer& P = S.prod;
     if (P.o == P.len) {
-        P.par ^= 1;
+        P.par = (P.par + 1) % kIds;
         P.o = 0;
         P.c = atomicAdd(counter, 1);
         S.chunk[P.par] = P.c;
@@ -380,6 +389,7 @@ __device__ __forceinline__ bool produce(BulkShared& S, int u, const ChunkGeo& cg
     return true;
 }
 
+template <int kIds>  // 2, or kChunkIds for small matches
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     match_tiles_fp32_bulk(const float2* __restrict__ pp, const int32_t* __restrict__ pperm,
                           const unsigned long long* __restrict__ pmask, int64_t np_cap, const int64_t* d_np,
@@ -407,7 +417,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         mbar_fence_init();
         S.failed = 0;
         S.end_item = INT_MAX;
-        S.cg = chunk_geo(W, ctas, chunks_per_cta);
+        S.cg = chunk_geo(W, ctas, chunks_per_cta, kIds > 2);
     }
     __syncthreads();
     int issued = 0;  // meaningful in thread 0: local items whose copies were issued
@@ -425,12 +435,12 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
             bulk_g2s(S.pperm, pperm + rt0 * kTile, kPermBytes, &S.bar_p);
             bulk_g2s(S.pm, pmask + (rt0 & ~1), 16, &S.bar_p);
             for (int u = 0; u < kStages; ++u)
-                if (!produce(S, u, cg, W, nqt, counter, qn, qperm, qmask, issued)) break;
+                if (!produce<kIds>(S, u, cg, W, nqt, counter, qn, qperm, qmask, issued)) break;
         }
     }
     __syncthreads();
     if (read_end(S) == 0) return;
-    // this thread's view of the current item: chunk id and parity, items
+    // this thread's view of the current item: chunk id and its place, items
     // left in the chunk after it, row and column tile, ring stage and phase
     int cid = S.chunk[0];
     int kpar = 0;
@@ -563,7 +573,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         }
         __syncthreads();  // (2) stage s, the source tile and colred are free
         if (failed) break;
-        if (tid == 0 && read_end(S) == INT_MAX) produce(S, t + kStages, cg, W, nqt, counter, qn, qperm, qmask, issued);
+        if (tid == 0 && read_end(S) == INT_MAX) produce<kIds>(S, t + kStages, cg, W, nqt, counter, qn, qperm, qmask, issued);
         // advance to the next item (its chunk id is known: it was produced
         // kStages items ago); a new row tile reloads the source tile
         if (t + 1 < read_end(S)) {
@@ -576,7 +586,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
                     rt1 = rt + 1;
                 }
             } else {
-                kpar ^= 1;
+                kpar = (kpar + 1) % kIds;
                 cid = S.chunk[kpar];
                 left = chunk_len(cg, cid) - 1;
                 const int64_t x1 = chunk_start(cg, cid);
@@ -615,7 +625,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 // original row.
 __global__ void __launch_bounds__(256) merge_segments(const kmx::RowBest* __restrict__ seg,
                                                       const int32_t* __restrict__ pperm, int ctas,
-                                                      int chunks_per_cta, int64_t np_cap,
+                                                      int chunks_per_cta, bool small, int64_t np_cap,
                                                       const int64_t* d_np, int64_t nq_cap, const int64_t* d_nq,
                                                       const unsigned long long* __restrict__ colbest,
                                                       kmx::RowBest* __restrict__ merged, int32_t* __restrict__ mflag)
@@ -627,7 +637,7 @@ __global__ void __launch_bounds__(256) merge_segments(const kmx::RowBest* __rest
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < np; i += (int64_t)gridDim.x * 256) {
         kmx::RowBest r{INFINITY, 0x7fffffff, INFINITY};
         if (W > 0) {
-            const ChunkGeo cg = chunk_geo(W, ctas, chunks_per_cta);
+            const ChunkGeo cg = chunk_geo(W, ctas, chunks_per_cta, small);
             const int64_t rt = i / kTile;
             const int64_t cf = chunk_of(cg, rt * nqt), cl = chunk_of(cg, rt * nqt + nqt - 1);
             r = seg[(cf + rt) * kTile + (i % kTile)];
@@ -692,7 +702,10 @@ int max_ctas(int sm_count) { return kCtasPerSm * sm_count; }
 cudaError_t set_smem_attr()
 {
     return kmx_once_per_device(kmx_attr_fp32_bulk, [] {
-        return cudaFuncSetAttribute(match_tiles_fp32_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        const cudaError_t e = cudaFuncSetAttribute(
+            match_tiles_fp32_bulk<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BulkShared));
+        if (e) return e;
+        return cudaFuncSetAttribute(match_tiles_fp32_bulk<kChunkIds>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)sizeof(BulkShared));
     });
 }
@@ -724,7 +737,7 @@ cudaError_t kmx_match_fp32_bulk_launch(kmx_ctx* ctx, const float* dp, const int3
     cudaError_t e = set_smem_attr();
     if (e) return e;
     int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, match_tiles_fp32_bulk, kThreads,
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, match_tiles_fp32_bulk<2>, kThreads,
                                                            sizeof(BulkShared))))
         return e;
     const int want = ctx->match_ctas_per_sm > 0 ? ctx->match_ctas_per_sm : kCtasPerSm;
@@ -740,13 +753,15 @@ cudaError_t kmx_match_fp32_bulk_launch(kmx_ctx* ctx, const float* dp, const int3
     KMX_COUNT_LAUNCH();
     place_pack<<<small_grid, 256, 0, st>>>(b.sort);
     KMX_COUNT_LAUNCH();
-    match_tiles_fp32_bulk<<<ctas, kThreads, sizeof(BulkShared), st>>>(
+    const bool small = tiles_of(np_cap) * tiles_of(nq_cap) < (int64_t)kSmallPairs * ctas;
+    auto* tiles = small ? match_tiles_fp32_bulk<kChunkIds> : match_tiles_fp32_bulk<2>;
+    tiles<<<ctas, kThreads, sizeof(BulkShared), st>>>(
         static_cast<const float2*>(b.sort.packed[0]), b.sort.perm[0], b.sort.mask[0], np_cap, d_np,
         static_cast<const float*>(b.sort.packed[1]), b.sort.perm[1], b.sort.mask[1], nq_cap, d_nq, ctas, cpc,
         b.chunk_counter, b.seg, s.colbest, ctx->d_err);
     KMX_COUNT_LAUNCH();
     merge_segments<<<kmx_stride_blocks(np_cap, 256, ctx->sm_count), 256, 0, st>>>(
-        b.seg, b.sort.perm[0], ctas, cpc, np_cap, d_np, nq_cap, d_nq, s.colbest, s.merged, s.mflag);
+        b.seg, b.sort.perm[0], ctas, cpc, small, np_cap, d_np, nq_cap, d_nq, s.colbest, s.merged, s.mflag);
     if ((e = cudaGetLastError())) return e;
     return kmx::match_emit(ctx, s, np_cap, d_np, vp, vq, out, cap, n_out);
 }
