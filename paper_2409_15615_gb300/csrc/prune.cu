@@ -40,7 +40,8 @@ constexpr uint32_t kSpinLimit = 1u << 24;
 constexpr int kMaxRounds = 1 << 16;
 constexpr int kCoreThreads = 1024;
 constexpr int kCoreWarps = kCoreThreads / 32;
-constexpr int kPasses = 4;                  // passes between two grid barriers
+constexpr int kSyncGen = 64;                // words from the arrivals, which the pollers of the generation leave alone
+constexpr int kPasses = 3;                  // passes between two grid barriers
 constexpr size_t kCoreSmem = 136 * 1024;    // snapshot, vertex states and neighbour lists of a kcore CTA
 
 struct PruneScratch {
@@ -57,7 +58,7 @@ struct PruneScratch {
     float4* pb;               // [n_tau] target end point
     uint32_t* adj;            // [n_tau][words]
     uint16_t* core;           // [n_tau, padded to 8] working values
-    uint32_t* sync;           // [2] barrier arrivals (changed blocks in the high half), barrier generation
+    uint32_t* sync;           // barrier arrivals (changed blocks in the high half); at [kSyncGen] its generation
 };
 
 __device__ __forceinline__ int64_t corr_count(const int64_t* d_n, int64_t cap)
@@ -245,10 +246,10 @@ __device__ bool grid_barrier(uint32_t* sync, uint32_t nblocks, uint32_t round, b
             seen = want | (sum >> 16 ? 0x80000000u : 0u);
             atomicExch(sync, 0u);
             __threadfence();
-            atomicExch(sync + 1, seen);
+            atomicExch(sync + kSyncGen, seen);
         } else {
             uint32_t it = 0;
-            while (((seen = ld_volatile(sync + 1)) & 0x7fffffffu) != want) {
+            while (((seen = ld_volatile(sync + kSyncGen)) & 0x7fffffffu) != want) {
                 if (++it > kSpinLimit) {
                     seen = 0xffffffffu;
                     break;
@@ -273,28 +274,51 @@ struct CoreVertex {
     int32_t start;  // of the neighbour list in the warp's part, -1: the list did not fit
 };
 
-// number of neighbours u of the vertex with snap[u] >= h (warp-wide, every lane
-// gets it): over its list, or over its bit row
-__device__ __forceinline__ int count_ge(const uint16_t* list, int deg, const uint32_t* __restrict__ row, int words,
-                                        const uint16_t* snap, int h)
-{
-    const int lane = threadIdx.x & 31;
-    int cnt = 0;
-    if (list) {
+// The values of a vertex's neighbours for the counts of one visit: per lane in
+// registers up to 32 kHeld neighbours, else read again for every count, from the
+// list or by the bit row.
+constexpr int kHeld = 16;
+struct Neighbours {
+    int held[kHeld];
+    const uint16_t* list;
+    const uint32_t* row;
+    const uint16_t* snap;
+    int deg, words;
+
+    __device__ __forceinline__ void load()
+    {
+        const int lane = threadIdx.x & 31;
+        if (!list || deg > 32 * kHeld) return;
+#pragma unroll
+        for (int e = 0; e < kHeld; ++e)
+            if (32 * e < deg) held[e] = 32 * e + lane < deg ? snap[list[32 * e + lane]] : -1;
+    }
+
+    // number of neighbours with a value >= h > 0 (warp-wide, every lane gets it)
+    __device__ __forceinline__ int count_ge(int h) const
+    {
+        const int lane = threadIdx.x & 31;
+        int cnt = 0;
+        if (list && deg <= 32 * kHeld) {
+#pragma unroll
+            for (int e = 0; e < kHeld; ++e)
+                if (32 * e < deg) cnt += held[e] >= h;
+        } else if (list) {
 #pragma unroll 4
-        for (int e = lane; e < deg; e += 32) cnt += snap[list[e]] >= h;
-    } else {
-        for (int w = lane; w < words; w += 32) {
-            uint32_t bits = row[w];
-            while (bits) {
-                const int e = __ffs(bits) - 1;
-                bits &= bits - 1;
-                cnt += snap[w * 32 + e] >= h;
+            for (int e = lane; e < deg; e += 32) cnt += snap[list[e]] >= h;
+        } else {
+            for (int w = lane; w < words; w += 32) {
+                uint32_t bits = row[w];
+                while (bits) {
+                    const int e = __ffs(bits) - 1;
+                    bits &= bits - 1;
+                    cnt += snap[w * 32 + e] >= h;
+                }
             }
         }
+        return __reduce_add_sync(0xffffffffu, cnt);
     }
-    return __reduce_add_sync(0xffffffffu, cnt);
-}
+};
 
 // One warp per vertex (per_warp of them at most), whose neighbour list it keeps
 // in shared memory as 16-bit indices.  A pass reads all values (2 n bytes from
@@ -303,7 +327,9 @@ __device__ __forceinline__ int count_ge(const uint16_t* list, int deg, const uin
 // (a round without a change saw the same values in all its passes).  What
 // bounds it: the L2 round trip of a pass and the barrier's.  Before, a pass took
 // vertices from a global counter, walked 32-bit rows in L2 and ended in a
-// barrier: 3000 vertices of 160 neighbours took 1042 us, now 263 us.
+// barrier: 3000 vertices of 160 neighbours took 1042 us; with lists and four
+// passes to a barrier 263 us, with the values of a visit held in registers and three passes
+// 245 us.
 __global__ void __launch_bounds__(kCoreThreads, 1) kcore(const int64_t* d_n_sel, int32_t words, int32_t per_warp,
                                                          int32_t list_len, PruneScratch s,
                                                          int32_t* __restrict__ core_out, int32_t* __restrict__ kmax_out,
@@ -370,16 +396,21 @@ __global__ void __launch_bounds__(kCoreThreads, 1) kcore(const int64_t* d_n_sel,
             for (int k = 0, v = v0; v < n; ++k, v += step) {
                 const CoreVertex x = vert[k];
                 if (x.c == 0) continue;
-                const uint32_t* row = s.adj + (int64_t)v * words;
-                const uint16_t* nb = x.start >= 0 ? list + x.start : nullptr;
+                Neighbours nb;
+                nb.list = x.start >= 0 ? list + x.start : nullptr;
+                nb.row = s.adj + (int64_t)v * words;
+                nb.snap = snap;
+                nb.deg = x.deg;
+                nb.words = words;
+                nb.load();
                 // count_ge falls as h grows: with `lo` values >= c, at least
                 // `lo` are >= lo
-                int lo = count_ge(nb, x.deg, row, words, snap, x.c);
+                int lo = nb.count_ge(x.c);
                 if (lo >= x.c) continue;
                 int hi = x.c - 1;
                 while (lo < hi) {
                     const int mid = (lo + hi + 1) >> 1;
-                    if (count_ge(nb, x.deg, row, words, snap, mid) >= mid)
+                    if (nb.count_ge(mid) >= mid)
                         lo = mid;
                     else
                         hi = mid - 1;
@@ -431,7 +462,7 @@ __global__ void __launch_bounds__(kCoreThreads, 1) kcore(const int64_t* d_n_sel,
 
 int32_t words_for(int32_t n_tau) { return (n_tau + 31) / 32; }
 
-size_t zero_bytes() { return sizeof(int32_t) * (kBuckets + 2 + 2); }
+size_t zero_bytes() { return sizeof(int32_t) * (kBuckets + 2 + kSyncGen + 1); }
 
 PruneScratch carve(void* base, int64_t cap, int32_t n_tau, size_t* total)
 {
