@@ -282,65 +282,73 @@ __global__ void __launch_bounds__(kCentroidThreads) vox_centroid(const float* __
 // scanner): the lanes split the members, the exponent ranges and the integer
 // sums are combined with shuffles (integer addition is exact in any order);
 // a voxel that fails the exponent test is summed in input order by lane 0.
+// A warp's lanes look at 32 voxels at a time, far apart (big voxels are
+// neighbours in the output order): one voxel per warp and step took 33 us to
+// find that 300k voxels hold few big ones, this form 10 us.
 __global__ void __launch_bounds__(kThreads) vox_centroid_big(const float* __restrict__ xyz, int stride, int64_t n,
                                                             VoxScratch s, float4* __restrict__ out, int64_t cap)
 {
     const int lane = threadIdx.x & 31;
     const int64_t nv = min(s.oidx[n], cap);
     const int64_t warps = (int64_t)gridDim.x * (kThreads / 32);
-    for (int64_t o = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5; o < nv; o += warps) {
-        const int64_t b = s.vstart[o];
-        const int L = (int)(s.vstart[o + 1] - b);
-        if (L <= kBigVoxel) continue;
-        const int32_t* m = s.members + b;
-        int emin[3] = {255, 255, 255}, emax[3] = {0, 0, 0};
-        bool odd = false;
-        for (int e = lane; e < L; e += 32) {
-            const float* p = xyz + (int64_t)__ldg(m + e) * stride;
-            exp_range(p[0], emin[0], emax[0], odd);
-            exp_range(p[1], emin[1], emax[1], odd);
-            exp_range(p[2], emin[2], emax[2], odd);
-        }
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-#pragma unroll
-            for (int sh = 16; sh >= 1; sh >>= 1) {
-                emin[a] = min(emin[a], __shfl_xor_sync(0xffffffffu, emin[a], sh));
-                emax[a] = max(emax[a], __shfl_xor_sync(0xffffffffu, emax[a], sh));
-            }
-        }
-        odd = __any_sync(0xffffffffu, odd);
-        const int lg = 32 - __clz(L - 1);  // ceil(log2 L), L > 32
-        bool exact = !odd;
-        for (int a = 0; a < 3; ++a)
-            if (emax[a] >= emin[a] && emax[a] - emin[a] > 29 - lg) exact = false;
-        double sx = 0.0, sy = 0.0, sz = 0.0;
-        if (exact) {
-            long long ix = 0, iy = 0, iz = 0;
+    const int64_t warp = ((int64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
+    for (int64_t base = warp; base < nv; base += 32 * warps) {
+        const int64_t mine = base + lane * warps;
+        const bool big = mine < nv && s.vstart[mine + 1] - s.vstart[mine] > kBigVoxel;
+        for (unsigned todo = __ballot_sync(0xffffffffu, big); todo; todo &= todo - 1) {
+            const int64_t o = base + (int64_t)(__ffs(todo) - 1) * warps;
+            const int64_t b = s.vstart[o];
+            const int L = (int)(s.vstart[o + 1] - b);
+            const int32_t* m = s.members + b;
+            int emin[3] = {255, 255, 255}, emax[3] = {0, 0, 0};
+            bool odd = false;
             for (int e = lane; e < L; e += 32) {
                 const float* p = xyz + (int64_t)__ldg(m + e) * stride;
-                ix += scaled_int(p[0], emin[0]);
-                iy += scaled_int(p[1], emin[1]);
-                iz += scaled_int(p[2], emin[2]);
+                exp_range(p[0], emin[0], emax[0], odd);
+                exp_range(p[1], emin[1], emax[1], odd);
+                exp_range(p[2], emin[2], emax[2], odd);
             }
 #pragma unroll
-            for (int sh = 16; sh >= 1; sh >>= 1) {
-                ix += __shfl_xor_sync(0xffffffffu, ix, sh);
-                iy += __shfl_xor_sync(0xffffffffu, iy, sh);
-                iz += __shfl_xor_sync(0xffffffffu, iz, sh);
+            for (int a = 0; a < 3; ++a) {
+#pragma unroll
+                for (int sh = 16; sh >= 1; sh >>= 1) {
+                    emin[a] = min(emin[a], __shfl_xor_sync(0xffffffffu, emin[a], sh));
+                    emax[a] = max(emax[a], __shfl_xor_sync(0xffffffffu, emax[a], sh));
+                }
             }
-            sx = scaled_sum(ix, emin[0]);
-            sy = scaled_sum(iy, emin[1]);
-            sz = scaled_sum(iz, emin[2]);
-        } else if (lane == 0) {
-            ordered_sum(xyz, stride, m, L, s.run + b, sx, sy, sz);
+            odd = __any_sync(0xffffffffu, odd);
+            const int lg = 32 - __clz(L - 1);  // ceil(log2 L), L > 32
+            bool exact = !odd;
+            for (int a = 0; a < 3; ++a)
+                if (emax[a] >= emin[a] && emax[a] - emin[a] > 29 - lg) exact = false;
+            double sx = 0.0, sy = 0.0, sz = 0.0;
+            if (exact) {
+                long long ix = 0, iy = 0, iz = 0;
+                for (int e = lane; e < L; e += 32) {
+                    const float* p = xyz + (int64_t)__ldg(m + e) * stride;
+                    ix += scaled_int(p[0], emin[0]);
+                    iy += scaled_int(p[1], emin[1]);
+                    iz += scaled_int(p[2], emin[2]);
+                }
+#pragma unroll
+                for (int sh = 16; sh >= 1; sh >>= 1) {
+                    ix += __shfl_xor_sync(0xffffffffu, ix, sh);
+                    iy += __shfl_xor_sync(0xffffffffu, iy, sh);
+                    iz += __shfl_xor_sync(0xffffffffu, iz, sh);
+                }
+                sx = scaled_sum(ix, emin[0]);
+                sy = scaled_sum(iy, emin[1]);
+                sz = scaled_sum(iz, emin[2]);
+            } else if (lane == 0) {
+                ordered_sum(xyz, stride, m, L, s.run + b, sx, sy, sz);
+            }
+            if (lane == 0) {
+                const double c = (double)L;
+                out[o] = make_float4(__double2float_rn(__ddiv_rn(sx, c)), __double2float_rn(__ddiv_rn(sy, c)),
+                                     __double2float_rn(__ddiv_rn(sz, c)), 0.0f);
+            }
+            __syncwarp();
         }
-        if (lane == 0) {
-            const double c = (double)L;
-            out[o] = make_float4(__double2float_rn(__ddiv_rn(sx, c)), __double2float_rn(__ddiv_rn(sy, c)),
-                                 __double2float_rn(__ddiv_rn(sz, c)), 0.0f);
-        }
-        __syncwarp();
     }
 }
 
@@ -373,7 +381,7 @@ cudaError_t kmx_voxelize_launch(kmx_ctx* ctx, const float* xyz, int64_t n, const
     KMX_COUNT_LAUNCH();
     vox_number<<<nb, kThreads, 0, st>>>(n, d_n, s, cap, n_out, ctx->d_err);
     // member offsets per output voxel: scan of the counts vox_number left in `flag`
-    if ((e = kmx_scan_i32(ctx, s.flag, n, n_out, s.vstart))) return e;
+    if ((e = kmx_scan_i32_live(ctx, s.flag, n, n_out, s.vstart))) return e;
     KMX_COUNT_LAUNCH();
     vox_scatter<<<nb, kThreads, 0, st>>>(n, d_n, s, assign);
     KMX_COUNT_LAUNCH();
