@@ -1141,9 +1141,9 @@ __device__ __forceinline__ void load_row(const float* __restrict__ row, bool val
 //      path's arithmetic): its second-smallest d2 over distinct columns is
 //      an upper bound of the row's d(2); the columns with distance <= d2
 //      are its first candidates (cnt[row] = their number), and ub[row] = d2.
-// near[rt] is the tile cs.
+// near[rt] is the tile cs.  Only the first `most` columns of cs are compared.
 __device__ __forceinline__ void plan_nearest(PlanShared& S, const PlanDir& D, const int64_t rt, const int64_t rows,
-                                             const int64_t cols)
+                                             const int64_t cols, const int most)
 {
     float x[KMX_DESC_DIM];
     float(*ys)[kCenterStride] = S.ysc;
@@ -1195,7 +1195,7 @@ __device__ __forceinline__ void plan_nearest(PlanShared& S, const PlanDir& D, co
     const int64_t cs = S.cs;
     {
         const int64_t yp = cs * kTN + tid;
-        const bool yv = yp < cols;
+        const bool yv = yp < cols && tid < most;
         const float* yr = yv ? D.Y + (int64_t)D.permY[yp] * KMX_DESC_STRIDE : nullptr;
 #pragma unroll
         for (int h = 0; h < kCenterStride; ++h) ys[tid][h] = (yv && h < KMX_DESC_DIM) ? -__ldg(yr + h) : 0.f;
@@ -1208,7 +1208,7 @@ __device__ __forceinline__ void plan_nearest(PlanShared& S, const PlanDir& D, co
     // compared again (with the same arithmetic, so the same values) and those
     // within d2 become candidates.  More than kPlanRec records: a second
     // pass over the whole tile.
-    const int ncol = (int)min((int64_t)kTN, cols - cs * kTN);
+    const int ncol = (int)min((int64_t)most, cols - cs * kTN);
     float d2 = INFINITY;
     if (valid) {
         // the exact path's arithmetic: x + (-y) per dimension, one fused
@@ -1438,7 +1438,9 @@ __device__ __forceinline__ void plan_list(PlanShared& S, const PlanDir& D, const
 }
 
 // First candidates and bounds of both sides' rows in one launch (one tail
-// instead of two): CTAs take row tiles from a counter (*next, zeroed before the
+// instead of two; two columns for a target row, whose bound that matters comes
+// from the source rows; all 128 of them took 415 us against 298 us at 302548 x
+// 287858 rows): CTAs take row tiles from a counter (*next, zeroed before the
 // launch), first those of direction a, then those of b.
 __global__ void __launch_bounds__(kTM) tc_near(PlanDir a, PlanDir b, int* __restrict__ next)
 {
@@ -1453,9 +1455,9 @@ __global__ void __launch_bounds__(kTM) tc_near(PlanDir a, PlanDir b, int* __rest
         __syncthreads();  // S.next is read before thread 0 takes the next tile
         if (k >= ta + tb) break;
         if (k < ta)
-            plan_nearest(S, a, k, na, nb);
+            plan_nearest(S, a, k, na, nb, kTN);
         else
-            plan_nearest(S, b, k - ta, nb, na);
+            plan_nearest(S, b, k - ta, nb, na, 2);
         __syncthreads();  // the next tile rewrites the shared arrays
     }
 }
