@@ -13,7 +13,8 @@
 //                     bucket's, after the buckets below; ranks < N_tau give
 //                     the selection in ascending order, with both end points
 //                     gathered.
-//   graph_build       one 32-bit word of the adjacency bit matrix per thread:
+//   graph_build       32-bit words of the adjacency bit matrix, two per lane and
+//                     32 pair tests:
 //                     k ~ k' iff | |b_k - b_k'| - |a_k - a_k'| | <= 2 beta.  The
 //                     test runs in FP32; within a band around the threshold it
 //                     is decided again in FP64 as ((dx dx + dy dy) + dz dz),
@@ -177,7 +178,7 @@ __global__ void __launch_bounds__(kThreads) ratio_rank(const kmx_corr* __restric
 __device__ __forceinline__ float sqrt_approx(float x)
 {
     float y;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 
@@ -190,21 +191,35 @@ __device__ __forceinline__ bool edge_fp64(float4 a, float4 a2, float4 b, float4 
     return fabs(__dadd_rn(db, -da)) <= two_beta;
 }
 
-// Thread (v, w): bits u = 32 w .. 32 w + 31 of row v.
+// One warp per pair of 32-vertex blocks (bv >= bu): lane = vertex of bv, its
+// word for the block bu; the ballot over the lanes is the word of each vertex of
+// bu for the block bv, so every pair is tested once.  Bound by instruction issue
+// and the latency of the warp's uniform loads; 3000 vertices with every word
+// from its own 32 tests took 24 us, this form 15 us.
 __global__ void __launch_bounds__(kThreads) graph_build(int32_t n_tau, const int64_t* d_n_sel, double two_beta,
                                                        PruneScratch s, int32_t words)
 {
-    const int64_t nsel = *d_n_sel;
-    const int64_t total = nsel * words;
+    const int nsel = (int)*d_n_sel;
+    const int nb = (nsel + 31) / 32;
+    const int64_t total = (int64_t)nb * (nb + 1) / 2;
     const float tb = (float)two_beta;
-    // consecutive threads share w (the 32 end-point pairs they read are the same)
-    for (int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x; t < total; t += (int64_t)gridDim.x * kThreads) {
-        const int w = (int)(t / nsel), v = (int)(t - (int64_t)w * nsel);
-        const float4 a = s.pa[v], b = s.pb[v];
-        uint32_t bits = 0;
-        for (int e = 0; e < 32; ++e) {
-            const int u = w * 32 + e;
-            if (u >= nsel || u == v) continue;
+    const int lane = threadIdx.x & 31;
+    for (int64_t t = (int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); t < total;
+         t += (int64_t)gridDim.x * (kThreads / 32)) {
+        // t = bv (bv + 1) / 2 + bu
+        int bv = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+        while ((int64_t)(bv + 1) * (bv + 2) / 2 <= t) ++bv;
+        while ((int64_t)bv * (bv + 1) / 2 > t) --bv;
+        const int bu = (int)(t - (int64_t)bv * (bv + 1) / 2);
+        const int v = bv * 32 + lane;
+        const bool valid = v < nsel;
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 a = valid ? s.pa[v] : zero, b = valid ? s.pb[v] : zero;
+        uint32_t bits = 0, back = 0;
+        const int last = min(32, nsel - bu * 32);
+#pragma unroll 4
+        for (int e = 0; e < last; ++e) {
+            const int u = bu * 32 + e;
             const float4 a2 = s.pa[u], b2 = s.pb[u];
             const float ax = a.x - a2.x, ay = a.y - a2.y, az = a.z - a2.z;
             const float bx = b.x - b2.x, by = b.y - b2.y, bz = b.z - b2.z;
@@ -215,16 +230,15 @@ __global__ void __launch_bounds__(kThreads) graph_build(int32_t n_tau, const int
             // which halves the instructions of a pair, one more); decide again
             // in FP64 near the threshold
             const float band = 1e-5f * (1.0f + da + db);
-            bool on;
-            if (gap > band)
-                on = false;
-            else if (gap < -band)
-                on = true;
-            else
-                on = edge_fp64(a, a2, b, b2, two_beta);
+            bool on = gap < -band;
+            if (!on && !(gap > band)) on = edge_fp64(a, a2, b, b2, two_beta);
+            on = on && valid && u != v;
+            const unsigned all = __ballot_sync(0xffffffffu, on);
             bits |= (uint32_t)on << e;
+            if (lane == e) back = all;
         }
-        s.adj[(int64_t)v * words + w] = bits;
+        if (valid) s.adj[(int64_t)v * words + bu] = bits;
+        if (bu != bv && lane < last) s.adj[(int64_t)(bu * 32 + lane) * words + bv] = back;
     }
 }
 
@@ -337,6 +351,7 @@ __global__ void __launch_bounds__(kCoreThreads, 1) kcore(const int64_t* d_n_sel,
                                                          unsigned int* __restrict__ err)
 {
     const int n = (int)*d_n_sel;
+    const int n_words = (n + 31) / 32;  // of the row's `words` (graph_build writes no others)
     const uint32_t nblocks = gridDim.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // dynamic shared memory: the values at the start of a pass, the warps'
@@ -353,8 +368,8 @@ __global__ void __launch_bounds__(kCoreThreads, 1) kcore(const int64_t* d_n_sel,
     for (int k = 0, v = v0; v < n; ++k, v += step) {
         const uint32_t* row = s.adj + (int64_t)v * words;
         int deg = 0;
-        for (int w0 = 0; w0 < words; w0 += 32) {
-            uint32_t bits = w0 + lane < words ? row[w0 + lane] : 0u;
+        for (int w0 = 0; w0 < n_words; w0 += 32) {
+            uint32_t bits = w0 + lane < n_words ? row[w0 + lane] : 0u;
             const int mine = __popc(bits);
             int inc = mine;
 #pragma unroll
@@ -401,7 +416,7 @@ __global__ void __launch_bounds__(kCoreThreads, 1) kcore(const int64_t* d_n_sel,
                 nb.row = s.adj + (int64_t)v * words;
                 nb.snap = snap;
                 nb.deg = x.deg;
-                nb.words = words;
+                nb.words = n_words;
                 nb.load();
                 // count_ge falls as h grows: with `lo` values >= c, at least
                 // `lo` are >= lo
@@ -518,7 +533,7 @@ cudaError_t kmx_prune_launch(kmx_ctx* ctx, const kmx_corr* corr, int64_t cap, co
     ratio_rank<<<grid, kThreads, 0, st>>>(corr, n_tau, src4, tgt4, s, sel);
     const int32_t words = words_for(n_tau);
     KMX_COUNT_LAUNCH();
-    graph_build<<<grid, kThreads, 0, st>>>(n_tau, n_sel, 2.0 * beta, s, words);
+    graph_build<<<2 * grid, kThreads, 0, st>>>(n_tau, n_sel, 2.0 * beta, s, words);
     // one CTA per SM (co-resident under a cooperative launch: the rounds wait
     // on one another through the grid barrier)
     const unsigned kgrid = (unsigned)ctx->sm_count;
