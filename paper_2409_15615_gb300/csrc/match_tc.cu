@@ -6,9 +6,8 @@
 // |x|^2 + |y|^2 - 2 x.y loses the bits that d^2 needs when |x| |y| >> d^2;
 // the descriptors of plane points are near-duplicates (d^2 ~ 0.3 against
 // |x - mean|^2 ~ 10^3), so one global centre is not enough.  Rows that are
-// close in descriptor space are therefore put next to each other (a Morton
-// key over four statistics of the histograms, radix-sorted), every 128-row
-// tile gets its own centre c, and each tile pair is computed as
+// close in descriptor space are therefore put next to each other (a
+// principal-direction tree), every 128-row tile gets its own centre c, and each tile pair is computed as
 //     d^2(x, y) = |x - c_C|^2 + |y - c_C|^2 - 2 (x - c_C).(y - c_C)
 // with c_C the centre of the column tile: both factors of the product are
 // small exactly for the pairs whose ranking matters.
